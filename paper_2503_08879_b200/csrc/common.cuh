@@ -128,6 +128,8 @@ constexpr int kDecodeExtraClusters = 2;                                // cluste
 constexpr int kDecodeMaxTiles = 44;                                    // most 16-row tiles a CTA takes: its K tiles must all be resident, and a warp keeps the scores of six
 constexpr int kPartialStride = kMaxGroup * kHeadDim + 2 * kMaxGroup;   // floats per cluster result: O[8][128], m[8], l[8]
 
+constexpr int kStreamCtasPerSm = 2;                                    // CTAs of the stream kernel that fit on one SM
+
 struct DecodeParams {
   const uint16_t *q;       // [B, H_q, 128]
   const uint16_t *k_new;   // [B, H_kv, 128] or null
@@ -155,8 +157,9 @@ struct DeviceInfo {
 };
 cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStream_t stream);
 cudaError_t decode_setup(DeviceInfo *dev);   // one-time, with the device current
-void decode_geometry(int L, int heads, const DeviceInfo *dev, int *n_clusters, int *cluster_size, int *resident_tiles,
-                     int *smem_bytes);
+// returns the estimated us of a launch, 0 if there is none; `overlap`: the rows are requested ahead of the dependency wait
+float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int *n_clusters, int *cluster_size,
+                      int *resident_tiles, int *smem_bytes);
 
 // ---- status word -------------------------------------------------------------
 // One int32 in device memory per context, OR-ed into by the kernels, read by sagekv_status.

@@ -28,6 +28,7 @@
 // reached and the kernel ends; the output of such a launch is meaningless and the status word says so.
 #include <cooperative_groups.h>
 #include <cuda.h>
+#include <math.h>
 
 #include <mutex>
 
@@ -647,6 +648,7 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
 }  // namespace sagekv
 
 #include "decode_attn_tc.cuh"
+#include "decode_stream.cuh"
 
 namespace sagekv {
 
@@ -654,27 +656,26 @@ static size_t decode_tc_smem_bytes(int per_cta) {
   return 1024 + (size_t)((per_cta + 7) / 8) * kTcBlockBytes + (size_t)per_cta * kSlotBytes + sizeof(DecShared);
 }
 
+static_assert(kStreamCtasPerSm * (sizeof(StShared) + 1024) <= 233472, "two CTAs of the stream kernel fit on one SM");
 static_assert(1024 + (size_t)kDecodeSlots * kSlotBytes + sizeof(DecShared) <= 232448, "the staging area and the rest fit into 227 KB");
 static int decode_slots(int per_cta) { return 2 * per_cta < kDecodeSlots ? 2 * per_cta : kDecodeSlots; }
 static size_t decode_smem_bytes(int per_cta) {
   return 1024 + (size_t)decode_slots(per_cta) * kSlotBytes + sizeof(DecShared);
 }
 
-// How many clusters of `c` CTAs that take `tiles` tiles each can be on the device at once (a cluster must fit
-// into one GPC, so this is not n_sm / c: on this part 15 clusters of 8 whole-SM CTAs but 22 of 6).  Asked of the
-// runtime once per (device, size, tiles) and remembered.  0: unknown.
-static int g_cluster_cap[64][kDecodeMaxCluster + 1][kDecodeMaxTiles + 1];   // answer + 1; 0 = not asked yet
+// How many clusters of `c` CTAs of a kernel can be on the device at once (a cluster must fit into one GPC, so this is
+// not n_sm / c: on this part 15 clusters of 8 whole-SM CTAs but 22 of 6).  Asked of the runtime once per slot of the
+// caller's table and remembered there as answer + 1.  0: unknown.
 static std::mutex g_cap_mutex;
 
-static int cluster_capacity(int device, int c, int tiles) {
-  if (device < 0 || device >= 64 || c < 1 || c > kDecodeMaxCluster || tiles < 0 || tiles > kDecodeMaxTiles) return 0;
+template <typename Kernel>
+static int cluster_capacity(Kernel kernel, int threads, size_t smem, int c, int *slot) {
   std::lock_guard<std::mutex> lock(g_cap_mutex);
-  int &slot = g_cluster_cap[device][c][tiles];
-  if (slot == 0) {
+  if (*slot == 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(c * 64), 1, 1);
-    cfg.blockDim = dim3(kDecodeThreads, 1, 1);
-    cfg.dynamicSmemBytes = decode_smem_bytes(tiles);
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = c;
@@ -683,13 +684,32 @@ static int cluster_capacity(int device, int c, int tiles) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int nn = 0;
-    if (cudaOccupancyMaxActiveClusters(&nn, decode_attn_kernel<true>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&nn, kernel, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
       nn = 0;
     }
-    slot = nn + 1;
+    *slot = nn + 1;
   }
-  return slot - 1;
+  return *slot - 1;
+}
+
+static int resident_capacity(int device, int c, int tiles) {   // of decode_attn_kernel, `tiles` tiles per CTA
+  static int table[64][kDecodeMaxCluster + 1][kDecodeMaxTiles + 1];
+  if (device < 0 || device >= 64 || c < 1 || c > kDecodeMaxCluster || tiles < 0 || tiles > kDecodeMaxTiles) return 0;
+  return cluster_capacity(decode_attn_kernel<true>, kDecodeThreads, decode_smem_bytes(tiles), c, &table[device][c][tiles]);
+}
+
+static int stream_capacity(int device, int c) {                // of decode_stream_kernel, clusters of c CTAs
+  static int table[64][kStMaxCluster + 1];
+  if (device < 0 || device >= 64 || c < 1 || c > kStMaxCluster) return 0;
+  return cluster_capacity(decode_stream_kernel, kStThreads, sizeof(StShared), c, &table[device][c]);
+}
+
+// What moving the launch's rows takes next to a kernel's own time of `us` (the larger one dominates, and the other is
+// not hidden completely): fitted as the cube root of the sum of cubes.
+static float with_traffic(float us, int heads, int L) {
+  const float t = 1.f + (float)heads * (float)L * (4.f * kHeadDim) / 6.4e6f;   // 6.4 TB/s
+  return cbrtf(us * us * us + t * t * t);
 }
 
 cudaError_t decode_setup(DeviceInfo *dev) {
@@ -700,6 +720,9 @@ cudaError_t decode_setup(DeviceInfo *dev) {
   const cudaError_t e2 = cudaFuncSetAttribute(decode_attn_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)decode_smem_bytes(kDecodeMaxTiles));
   if (e2 != cudaSuccess) return e2;
+  cudaError_t e3 = cudaFuncSetAttribute(decode_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StShared));
+  if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(decode_stream_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of 16
+  if (e3 != cudaSuccess) return e3;
   return cudaFuncSetAttribute(decode_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)decode_tc_smem_bytes(kTcMaxTiles));
 }
 
@@ -710,32 +733,34 @@ cudaError_t decode_setup(DeviceInfo *dev) {
 // computes), which only works if the clusters of two launches fit on the device together, so the cluster sizes
 // are compared by a cost fitted to measurements (below).
 // (15 clusters of 8 whole-SM CTAs fit at once, 22 of 6, 26 of 5, 33 of 4.)
-void decode_geometry(int L, int heads, const DeviceInfo *dev, int *n_clusters, int *cs, int *per_cta_tiles, int *smem_bytes) {
+float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int *n_clusters, int *cs, int *per_cta_tiles,
+                      int *smem_bytes) {
   const int n_tiles = (L + 15) / 16;
   int c = 1;
   while (c < kDecodeBaseCluster && c * 2 <= n_tiles) c <<= 1;                   // cluster size 1, 2, 4 or 8
   int nc = (n_tiles + c * kDecodeMaxTiles - 1) / (c * kDecodeMaxTiles);          // the fewest clusters per head
-  if (dev != nullptr && heads > 0 && c == kDecodeBaseCluster) {
-    float best = 0.f;
+  float best = 0.f;
+  int best_waves = 1;
+  if (dev != nullptr && heads > 0) {
     int best_c = c, best_nc = nc;
     // up to kDecodeExtraClusters more clusters per head than needed: beyond one cluster the results are merged
     // through scratch anyway, and more, smaller clusters leave fewer V tiles waiting for a K slot
     for (int n_try = nc; n_try <= (nc > 1 ? nc + kDecodeExtraClusters : nc); ++n_try) {
-      for (int cand = kDecodeBaseCluster; cand >= 4; --cand) {
+      for (int cand = c; cand >= (c == kDecodeBaseCluster ? 4 : c); --cand) {
         const int per = (n_tiles + cand * n_try - 1) / (cand * n_try);
         if (per > kDecodeMaxTiles) continue;
-        const int cap = cluster_capacity(dev->device, cand, per);
+        const int cap = resident_capacity(dev->device, cand, per);
         if (cap <= 0) continue;
         // measured on this part (us per launch, batch 1 x 8 heads, L = 1025 / 2049 / 4097, clusters of 5 to 8):
         // 2.97 + 0.0445 per tile of a CTA; the same again per tile when the clusters of two launches do not fit
         // together (the copies are then issued on the critical path); 0.084 per V tile that has to wait for a K
-        // slot; 2.6 for the merge through scratch (L = 8193)
+        // slot; 3.4 for the merge through scratch (L = 8193, 1 and 8 heads)
         const int late = 2 * per > kDecodeSlots ? 2 * per - kDecodeSlots : 0;
         const int waves = (heads * n_try + cap - 1) / cap;                      // of one launch
         const float one = 2.97f + 0.0445f * (float)per * (2 * heads * n_try <= cap ? 1.f : 2.f) + 0.084f * (float)late +
-                          (n_try > 1 ? 2.6f : 0.f);
+                          (n_try > 1 ? 3.4f : 0.f);
         const float cost = (float)waves * one;
-        if (best == 0.f || cost < best) { best = cost; best_c = cand; best_nc = n_try; }
+        if (best == 0.f || cost < best) { best = cost; best_c = cand; best_nc = n_try; best_waves = waves; }
       }
     }
     c = best_c;
@@ -748,6 +773,33 @@ void decode_geometry(int L, int heads, const DeviceInfo *dev, int *n_clusters, i
   *cs = c;
   *per_cta_tiles = per_cta;
   *smem_bytes = (int)decode_smem_bytes(per_cta);
+  // without overlap: 3.9 + 0.14 per tile (the copies are issued on the critical path: L = 257 .. 4097, 1 to 16 heads)
+  if (best > 0.f && !overlap) best = (float)best_waves * (3.9f + 0.14f * (float)per_cta + (nc > 1 ? 3.4f : 0.f));
+  return best > 0.f ? with_traffic(best, heads, L) : 0.f;
+}
+
+// The best launch of decode_stream_kernel: CTAs per head, heads per CTA, and its cost in us (0: none).  Measured over
+// 1 to 600 heads and L = 257 .. 8193: 2.4 plus 0.6 per tile of a warp (the ring's three tiles per warp in flight against
+// the latency of a copy); 1.7 more when the launches do not overlap; up to 1.5 more when two launches' CTAs do
+// not fit on the device together; 0.8 per further head of a CTA; a second wave costs a whole time again.
+static float stream_geometry(int L, int heads, const DeviceInfo &dev, bool overlap, int *split, int *per_cta) {
+  const int n_tiles = (L + 15) / 16;
+  if ((int64_t)n_tiles * heads > (int64_t)1 << 30) return 0.f;
+  float best = 0.f;
+  for (int s = 1; s <= kStMaxCluster && s <= n_tiles; s <<= 1) {
+    const int cap = s == 1 ? kStreamCtasPerSm * dev.n_sm : s * stream_capacity(dev.device, s);
+    if (cap <= 0) continue;
+    const int per = s == 1 ? (heads + cap - 1) / cap : 1;
+    const int ctas = s == 1 ? (heads + per - 1) / per : heads * s;
+    const int waves = (ctas + cap - 1) / cap;
+    const int rounds = (per * ((n_tiles + s - 1) / s) + kStWarps - 1) / kStWarps;
+    float one = 2.4f + 0.6f * (float)rounds + 0.8f * (float)(per - 1);
+    if (!overlap) one += 1.7f;
+    float cost = with_traffic((float)waves * one, heads, L);
+    if (2 * ctas > cap) cost += 0.5f + (float)(2 * (ctas < cap ? ctas : cap) - cap) / (float)cap;
+    if (best == 0.f || cost < best) { best = cost; *split = s; *per_cta = per; }
+  }
+  return best;
 }
 
 // cuTensorMapEncodeTiled, looked up through the runtime (the library does not link against the driver)
@@ -785,33 +837,47 @@ static bool make_cache_map(CUtensorMap *map, const uint16_t *base, const DecodeP
 }
 
 cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStream_t stream) {
-  int n_clusters, cs, per_cta, smem;
-  decode_geometry(p.L, p.B * p.H_kv, &dev, &n_clusters, &cs, &per_cta, &smem);
+  int n_clusters, cs, per_cta, smem, split = 1, heads_per_cta = 1;
+  const bool overlap = p.pdl_mode == 2;
+  const float cost = decode_geometry(p.L, p.B * p.H_kv, &dev, overlap, &n_clusters, &cs, &per_cta, &smem);
+  const bool tc = p.variant == 2 && n_clusters == 1 && per_cta <= kTcMaxTiles;
+  // Caches that fill the SMs more than once, and long ones, are streamed; short ones are brought in whole.  (us per
+  // launch whole / streamed, overlapping: 8 heads x 2049 rows 4.1 / 4.7, 8 x 8193 11.0 / 9.4, 64 x 2049 17.4 / 13.4,
+  // 256 x 2049 84.8 / 42.8)
+  const float stream_cost = tc ? 0.f : stream_geometry(p.L, p.B * p.H_kv, dev, overlap, &split, &heads_per_cta);
+  const bool streamed = stream_cost > 0.f && cost > 0.f && stream_cost < cost;
   CUtensorMap map_k, map_v;
   if (!make_cache_map(&map_k, p.Kc, p) || !make_cache_map(&map_v, p.Vc, p)) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n_clusters * cs), (unsigned)p.H_kv, (unsigned)p.B);
-  cfg.blockDim = dim3(kDecodeThreads, 1, 1);
-  cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cs;
+  attr[0].val.clusterDim.x = streamed ? split : cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = p.pdl_mode > 0 ? 2 : 1;
+  if (streamed) {
+    const int heads = p.B * p.H_kv;
+    cfg.gridDim = dim3((unsigned)(split > 1 ? heads * split : (heads + heads_per_cta - 1) / heads_per_cta), 1, 1);
+    cfg.blockDim = dim3(kStThreads, 1, 1);
+    cfg.dynamicSmemBytes = sizeof(StShared);
+    return cudaLaunchKernelEx(&cfg, decode_stream_kernel, p, map_k, map_v, split, heads_per_cta);
+  }
+  cfg.gridDim = dim3((unsigned)(n_clusters * cs), (unsigned)p.H_kv, (unsigned)p.B);
+  cfg.blockDim = dim3(kDecodeThreads, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)smem;
   // the tensor-memory variant where it applies: one cluster per head, every tile resident twice over
-  if (p.variant == 2 && n_clusters == 1 && per_cta <= kTcMaxTiles) {
+  if (tc) {
     cfg.dynamicSmemBytes = decode_tc_smem_bytes(per_cta);
     return cudaLaunchKernelEx(&cfg, decode_attn_tc_kernel, p, map_k, map_v, per_cta);
   }
   // the short instance keeps three tiles' scores per warp and has every V tile resident from the start
   const bool is_long = 2 * per_cta > kDecodeSlots || per_cta > kQkGroup * kDecodeWarps;
   return is_long ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true>, p, map_k, map_v, decode_slots(per_cta))
-                                    : cudaLaunchKernelEx(&cfg, decode_attn_kernel<false>, p, map_k, map_v, decode_slots(per_cta));
+                 : cudaLaunchKernelEx(&cfg, decode_attn_kernel<false>, p, map_k, map_v, decode_slots(per_cta));
 }
 
 }  // namespace sagekv
