@@ -1,6 +1,6 @@
 """ctypes binding of libsagekv.so (include/sagekv.h).
 
-Argument marshalling only: every function below has the name and the meaning of
+Argument marshalling only (the hot calls' in C, csrc/marshal.cpp): every function below has the name and the meaning of
 the C entry point it calls, takes torch CUDA tensors for the device buffers and
 passes their pointers, strides and the current CUDA stream through.  Nothing is
 computed here, and there is no fallback: importing this module raises if the
@@ -22,6 +22,12 @@ if not os.path.exists(_LIB_PATH):
         f"{_LIB_PATH} is missing: build it with `python -m paper_2503_08879_b200.build` "
         "(nvcc, sm_100a). There is no CPU or PyTorch fallback.")
 lib = C.CDLL(_LIB_PATH)
+
+try:
+    from . import _marshal
+except ImportError as e:
+    raise ImportError("paper_2503_08879_b200/_marshal.so is missing: build it with "
+                      "`python -m paper_2503_08879_b200.build`") from e
 
 OK, ERR_INVALID, ERR_ALIGN, ERR_UNSUPPORTED, ERR_CUDA, ERR_NOMEM = 0, -1, -2, -3, -4, -5
 ERR_TOO_LARGE, ERR_TIMEOUT, ERR_BOUNDS, ERR_DEVICE = -6, -7, -8, -9
@@ -106,8 +112,23 @@ def _ptr(t):
     return None if t is None else C.c_void_p(t.data_ptr())
 
 
+try:        # the handle alone: torch.cuda.current_stream() builds a stream object first
+    _device_now, _stream_of_device = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+except AttributeError:
+    def _stream_handle() -> int:
+        return torch.cuda.current_stream().cuda_stream
+else:
+    def _stream_handle() -> int:
+        return _stream_of_device(_device_now())
+
+
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(_stream_handle())
+
+
+_marshal.bind(*(C.cast(f, _vp).value for f in (lib.sagekv_score, lib.sagekv_select_compact, lib.sagekv_decode_attn,
+                                               lib.sagekv_pool_scores, lib.sagekv_quest_bounds, lib.sagekv_select_topk)),
+              _stream_handle, C.ArgumentError)
 
 
 def _kv_strides(t: torch.Tensor) -> Strides:
@@ -136,8 +157,9 @@ def sagekv_destroy(ctx):
 
 
 def sagekv_score(ctx, q_last, K, n_ctx: int, n_init: int, n_recent: int, scores, scores_row_stride: int):
-    _check(lib.sagekv_score(ctx, _ptr(q_last), _ptr(K), _kv_strides(K), n_ctx, n_init, n_recent, _ptr(scores),
-                            scores_row_stride, _stream()), "sagekv_score", ctx)
+    code = _marshal.score(ctx, q_last, K, n_ctx, n_init, n_recent, scores, scores_row_stride)
+    if code:
+        _check(code, "sagekv_score", ctx)
 
 
 def sagekv_set_overlap(ctx, mode: int):
@@ -169,8 +191,9 @@ def sagekv_set_group_mode(ctx, mode: int):
 
 def sagekv_pool_scores(ctx, scores, scores_row_stride: int, n_ctx: int, n_init: int, n_recent: int, pooled,
                        pooled_row_stride: int):
-    _check(lib.sagekv_pool_scores(ctx, _ptr(scores), scores_row_stride, n_ctx, n_init, n_recent, _ptr(pooled),
-                                  pooled_row_stride, _stream()), "sagekv_pool_scores", ctx)
+    code = _marshal.pool_scores(ctx, scores, scores_row_stride, n_ctx, n_init, n_recent, pooled, pooled_row_stride)
+    if code:
+        _check(code, "sagekv_pool_scores", ctx)
 
 
 def sagekv_compact_window_rope(ctx, K_pre, V, n_ctx: int, n_init: int, n_recent: int, rope_theta: float, Kc, Vc,
@@ -186,13 +209,15 @@ def sagekv_quest_build(ctx, K, n_ctx: int, n_init: int, n_recent: int, kmin, kma
 
 
 def sagekv_quest_bounds(ctx, q, kmin, kmax, n_blocks: int, bounds, bounds_row_stride: int):
-    _check(lib.sagekv_quest_bounds(ctx, _ptr(q), _ptr(kmin), _ptr(kmax), n_blocks, _ptr(bounds), bounds_row_stride,
-                                   _stream()), "sagekv_quest_bounds", ctx)
+    code = _marshal.quest_bounds(ctx, q, kmin, kmax, n_blocks, bounds, bounds_row_stride)
+    if code:
+        _check(code, "sagekv_quest_bounds", ctx)
 
 
 def sagekv_select_topk(ctx, scores, scores_row_stride: int, n: int, k_q: int, idx):
-    _check(lib.sagekv_select_topk(ctx, _ptr(scores), scores_row_stride, n, k_q, _ptr(idx), _stream()),
-           "sagekv_select_topk", ctx)
+    code = _marshal.select_topk(ctx, scores, scores_row_stride, n, k_q, idx)
+    if code:
+        _check(code, "sagekv_select_topk", ctx)
 
 
 def sagekv_status(ctx) -> int:
@@ -215,14 +240,15 @@ def sagekv_score_static(shape: Shape, q_last, K, n_ctx: int, n_init: int, n_rece
 
 def sagekv_select_compact(ctx, scores, scores_row_stride: int, K, V, n_ctx: int, n_init: int, n_recent: int, k: int,
                           idx, Kc, Vc, state: CacheState):
-    _check(lib.sagekv_select_compact(ctx, _ptr(scores), scores_row_stride, _ptr(K), _ptr(V), _kv_strides(K), n_ctx,
-                                     n_init, n_recent, k, _ptr(idx), _ptr(Kc), _ptr(Vc), _kv_strides(Kc),
-                                     C.byref(state), _stream()), "sagekv_select_compact", ctx)
+    code = _marshal.select_compact(ctx, scores, scores_row_stride, K, V, n_ctx, n_init, n_recent, k, idx, Kc, Vc, state)
+    if code:
+        _check(code, "sagekv_select_compact", ctx)
 
 
 def sagekv_decode_attn(ctx, q, k_new, v_new, Kc, Vc, state: CacheState, out, lse=None):
-    _check(lib.sagekv_decode_attn(ctx, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(Kc), _ptr(Vc), _kv_strides(Kc),
-                                  C.byref(state), _ptr(out), _ptr(lse), _stream()), "sagekv_decode_attn", ctx)
+    code = _marshal.decode_attn(ctx, q, k_new, v_new, Kc, Vc, state, out, lse)
+    if code:
+        _check(code, "sagekv_decode_attn", ctx)
 
 
 class Layer:

@@ -6,12 +6,14 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsagekv.so")
 LIB_CHECKED = os.path.join(HERE, "libsagekv_checked.so")   # the same interface built with -DSAGEKV_CHECKS
+MARSHAL = os.path.join(HERE, "_marshal.so")                # argument marshalling of the Python binding's hot calls
 LIB_TRACE = os.path.join(HERE, "libsagekv_trace.so")       # built with -DSAGEKV_TRACE: timeline stamps in the decode kernel
 SOURCES = ["api.cu", "score.cu", "score_static.cu", "select_compact.cu", "decode_attn.cu", "variants.cu"]
 
@@ -23,17 +25,32 @@ def nvcc_path() -> str:
     raise RuntimeError("nvcc not found")
 
 
+def build_marshal(force: bool = False) -> str:
+    src = os.path.join(CSRC, "marshal.cpp")
+    deps = [src, os.path.join(ROOT, "include", "sagekv.h")]
+    if not force and os.path.exists(MARSHAL) and all(os.path.getmtime(d) <= os.path.getmtime(MARSHAL) for d in deps):
+        return MARSHAL
+    cxx = os.environ.get("CXX") or shutil.which("g++") or "c++"
+    cmd = [cxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
+           "-o", MARSHAL, src]
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("building the marshalling module failed:\n" + res.stdout + res.stderr)
+    return MARSHAL
+
+
 def needs_build(lib: str = LIB) -> bool:
     if not os.path.exists(lib):
         return True
     t = os.path.getmtime(lib)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "sagekv.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))] + [os.path.join(ROOT, "include", "sagekv.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
 def build(force: bool = False, verbose: bool = False, checks: bool = False, trace: bool = False) -> str:
     """checks=True builds libsagekv_checked.so: every global-memory index of the kernels is range-checked and a
     violation is reported through sagekv_status instead of being executed (load it with SAGEKV_LIB=<path>)."""
+    build_marshal(force)
     lib = LIB_TRACE if trace else (LIB_CHECKED if checks else LIB)
     if not force and not needs_build(lib):
         return lib

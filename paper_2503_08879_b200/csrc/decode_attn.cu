@@ -30,6 +30,7 @@
 #include <cuda.h>
 #include <math.h>
 
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -665,13 +666,12 @@ static size_t decode_smem_bytes(int per_cta) {
 
 // How many clusters of `c` CTAs of a kernel can be on the device at once (a cluster must fit into one GPC, so this is
 // not n_sm / c: on this part 15 clusters of 8 whole-SM CTAs but 22 of 6).  Asked of the runtime once per slot of the
-// caller's table and remembered there as answer + 1.  0: unknown.
-static std::mutex g_cap_mutex;
+// caller's table and remembered there as answer + 1 (two threads may both ask: they get the same answer).  0: unknown.
 
 template <typename Kernel>
-static int cluster_capacity(Kernel kernel, int threads, size_t smem, int c, int *slot) {
-  std::lock_guard<std::mutex> lock(g_cap_mutex);
-  if (*slot == 0) {
+static int cluster_capacity(Kernel kernel, int threads, size_t smem, int c, std::atomic<int> *slot) {
+  int known = slot->load(std::memory_order_relaxed);
+  if (known == 0) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(c * 64), 1, 1);
     cfg.blockDim = dim3((unsigned)threads, 1, 1);
@@ -688,19 +688,20 @@ static int cluster_capacity(Kernel kernel, int threads, size_t smem, int c, int 
       (void)cudaGetLastError();
       nn = 0;
     }
-    *slot = nn + 1;
+    known = nn + 1;
+    slot->store(known, std::memory_order_relaxed);
   }
-  return *slot - 1;
+  return known - 1;
 }
 
 static int resident_capacity(int device, int c, int tiles) {   // of decode_attn_kernel, `tiles` tiles per CTA
-  static int table[64][kDecodeMaxCluster + 1][kDecodeMaxTiles + 1];
+  static std::atomic<int> table[64][kDecodeMaxCluster + 1][kDecodeMaxTiles + 1];
   if (device < 0 || device >= 64 || c < 1 || c > kDecodeMaxCluster || tiles < 0 || tiles > kDecodeMaxTiles) return 0;
   return cluster_capacity(decode_attn_kernel<true>, kDecodeThreads, decode_smem_bytes(tiles), c, &table[device][c][tiles]);
 }
 
 static int stream_capacity(int device, int c) {                // of decode_stream_kernel, clusters of c CTAs
-  static int table[64][kStMaxCluster + 1];
+  static std::atomic<int> table[64][kStMaxCluster + 1];
   if (device < 0 || device >= 64 || c < 1 || c > kStMaxCluster) return 0;
   return cluster_capacity(decode_stream_kernel, kStThreads, sizeof(StShared), c, &table[device][c]);
 }
