@@ -109,33 +109,59 @@ __device__ __forceinline__ void find_bin_from_top(const uint32_t *hist, int nb, 
   __syncthreads();
 }
 
-// one warp copies one K row (lanes 0-15) and one V row (lanes 16-31), 16 bytes per lane
-__device__ __forceinline__ void copy_kv_row(const SelectParams &p, int b, int kvh, int64_t src_tok, int64_t dst_row,
-                                            int lane) {
-  const uint16_t *src = (lane < 16 ? p.K : p.V) + (int64_t)b * p.ks.batch_stride + (int64_t)kvh * p.ks.head_stride +
-                        src_tok * p.ks.token_stride;
-  uint16_t *dst = (lane < 16 ? p.Kc : p.Vc) + (int64_t)b * p.cs.batch_stride + (int64_t)kvh * p.cs.head_stride +
-                  dst_row * p.cs.token_stride;
-  const int piece = (lane & 15) * 8;
-  if (SAGEKV_OK_INDEX(p.status, src_tok >= 0 && src_tok < p.N && dst_row >= 0 &&
-                                    dst_row < (int64_t)p.S + (int64_t)p.G * p.k_q + p.R + 1))
-    st_v4(dst + piece, ld_stream_v4(src + piece));
-}
+// ---- the rows whose positions are known without the scores: sink, recent, last token ------------------------------
+// A kernel of their own where they are all there is to copy (no selection), and where a row cluster would have to move
+// several per warp: there they are launched ahead of the selection, which does not wait for them and leaves
+// the memory idle with its chain of barriers and scans, and run beside it on what two selection CTAs per SM leave of the
+// registers (8192) and of the shared memory.  A warp moves a row with 16 bytes per lane (K in lanes 0-15, V in lanes 16-31)
+// through a ring of its own in shared memory, 16 rows in flight, so 64 KB per SM.
+constexpr int kStaticThreads = 256;
+constexpr int kStaticStages = 4;          // of four rows
+constexpr int kStaticSmem = (kStaticThreads / 32) * kStaticStages * 4 * 512;
 
-// sink rows, recent rows and the last token: positions known without the scores
-__device__ void copy_static_rows(const SelectParams &p, int cta, int n_ctas) {
-  const int lane = threadIdx.x & 31;
-  const int per_head = p.S + p.R + 1;
-  const int items = p.B * p.H_kv * per_head;
-  const int n_warps = n_ctas * kSelWarps;
-  for (int it = cta * kSelWarps + (threadIdx.x >> 5); it < items; it += n_warps) {
-    const int bk = it / per_head, r = it - bk * per_head;
-    const int b = bk / p.H_kv, kvh = bk - b * p.H_kv;
-    const int64_t src_tok = r < p.S ? r : (int64_t)p.E + r;                 // S + E + (r - S)
-    const int64_t dst_row = r < p.S ? r : (int64_t)p.G * p.k_q + r;         // S + G*k_q + (r - S)
-    copy_kv_row(p, b, kvh, src_tok, dst_row, lane);
+__global__ void __launch_bounds__(kStaticThreads, 8) copy_static_kernel(const SelectParams p, int alone) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  // (dependent launches: the selection that follows must find its inputs complete as soon as it starts)
+  if (p.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per_head = p.S + p.R + 1, groups = (per_head + 3) >> 2, items = p.B * p.H_kv * groups;
+  const int n_warps = (int)gridDim.x * (kStaticThreads / 32);
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem_raw) + (uint32_t)(warp * kStaticStages * 2048 + lane * 16);
+  const uint16_t *src0 = (lane < 16 ? p.K : p.V) + (lane & 15) * 8;
+  uint16_t *dst0 = (lane < 16 ? p.Kc : p.Vc) + (lane & 15) * 8;
+  auto issue = [&](int it, int stage) {
+    if (it < items) {
+      const int bk = it / groups, r0 = (it - bk * groups) * 4, b = bk / p.H_kv;
+      const uint16_t *src = src0 + (int64_t)b * p.ks.batch_stride + (int64_t)(bk - b * p.H_kv) * p.ks.head_stride;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int r = r0 + u, tok = r < p.S ? r : p.E + r;                   // S + E + (r - S)
+        if (r < per_head && SAGEKV_OK_INDEX(p.status, tok >= 0 && tok < p.N))
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ring + (uint32_t)(stage * 2048 + u * 512)),
+                       "l"(src + (int64_t)tok * p.ks.token_stride) : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  int it = blockIdx.x * (kStaticThreads / 32) + warp, stage = 0;
+#pragma unroll
+  for (int s = 0; s < kStaticStages; ++s) issue(it + s * n_warps, s);
+  for (; it < items; it += n_warps) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kStaticStages - 1) : "memory");   // every lane reads only what it copied itself
+    const int bk = it / groups, r0 = (it - bk * groups) * 4, b = bk / p.H_kv;
+    uint16_t *dst = dst0 + (int64_t)b * p.cs.batch_stride + (int64_t)(bk - b * p.H_kv) * p.cs.head_stride;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = r0 + u, row = r < p.S ? r : p.G * p.k_q + r;             // S + G*k_q + (r - S)
+      uint4 v;
+      asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(ring + (uint32_t)(stage * 2048 + u * 512)));
+      if (r < per_head) st_v4(dst + (int64_t)row * p.cs.token_stride, v);
+    }
+    issue(it + kStaticStages * n_warps, stage);
+    if (++stage == kStaticStages) stage = 0;
   }
-  if (cta == 0 && threadIdx.x == 0) *p.d_step = 0;
+  if (alone && blockIdx.x == 0 && threadIdx.x == 0) *p.d_step = 0;
 }
 
 // Geometry shared by the two paths
@@ -687,8 +713,10 @@ __device__ void general_select(cg::cluster_group &cluster, SelShared &sh, const 
 
 // kAhead: the instance for launches that start from a trusted candidate list with the dependency wait put off
 // (eight rows in flight per warp, which the other instance has no registers for).
+// (The launch bound of the other instance is 64 threads more than it has: that leaves it 56 registers, and the
+// static rows' kernel the room to run beside two of its CTAs.)
 template <bool kAhead>
-__global__ void __launch_bounds__(kSelThreads, 2) select_compact_kernel(const SelectParams p, int n_rows, int chunk,
+__global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) select_compact_kernel(const SelectParams p, int behind_static, int chunk,
                                                                       int resident, int list_cap, int cand_cap,
                                                                       int try_fast, int64_t sketch_off, int64_t list_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -703,10 +731,12 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_compact_kernel(const Se
   // complete (a request to bring the candidate list into L2 changes nothing a program can observe).  Mode 2 (the
   // caller vouches that the predecessor writes none of this call's inputs) puts the wait off until the first
   // write: selection and the first round of row loads run ahead of it, on the candidate-list path.
-  bool waited = p.pdl == 0;
+  // behind_static: the predecessor is this call's copy_static_kernel, which has found the inputs complete: nothing
+  // here depends on it, but this kernel's end stands for the whole call's, so it waits before it ends.
+  bool waited = p.pdl == 0 || behind_static;
   if (p.pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (p.pdl == 1 || (p.pdl == 2 && (list_off < 0 || cid >= n_rows))) {
-    if (list_off >= 0 && cid < n_rows) {
+  if (!waited && (p.pdl == 1 || list_off < 0)) {
+    if (list_off >= 0) {
       const char *lines = reinterpret_cast<const char *>(p.scores + (int64_t)cid * p.row_stride + list_off);
       const int n_lines = (kListTagWords * 4 + cand_cap * 8 + 127) >> 7;
       const int mine = rank + (int)threadIdx.x * cs;
@@ -716,10 +746,6 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_compact_kernel(const Se
     waited = true;
   }
   SAGEKV_STAMP(1);
-  if (cid >= n_rows) {   // whole cluster takes this branch together; it touches no peer's memory
-    copy_static_rows(p, (cid - n_rows) * cs + rank, (gridDim.x / cs - n_rows) * cs);
-    return;
-  }
 
   cluster.barrier_arrive();   // completed below: every CTA of the cluster runs before anyone writes into a peer
   SelShared &sh = *reinterpret_cast<SelShared *>(smem_raw);
@@ -856,7 +882,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_compact_kernel(const Se
                        ((int64_t)p.S + (int64_t)j * p.k_q) * p.cs.token_stride + (lane & 15) * 8;
   // The sink, recent and last rows of the KV head (positions known without the scores) are shared out over the
   // warps of the head's G clusters, at most one row per warp per round, loaded together with the first batch.
-  const int n_static = gather ? p.S + p.R + 1 : 0;
+  const int n_static = gather && !behind_static ? p.S + p.R + 1 : 0;
   const int static_stride = p.G * cs * kSelWarps;
   int sr = (j * cs + rank) * kSelWarps + warp;           // this warp's first static row
   constexpr int kRows = kAhead ? 8 : 4;                    // rows a warp has in flight: all loads issued before the stores
@@ -896,7 +922,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_compact_kernel(const Se
       sr += static_stride;
     }
   }
-  if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");   // a warp without a round of the loop
+  if (!waited || behind_static) asm volatile("griddepcontrol.wait;" ::: "memory");   // (not waited: a warp without a round of the loop)
   if (idx_deferred)                                        // every thread is here, and past the wait
     for (int i = tid; i < n_list_all; i += kSelThreads) {
       const int2 sp = c.list[i];
@@ -1044,7 +1070,9 @@ static size_t select_smem_bytes(int chunk, int list_cap, int cand_cap, int share
 }
 
 cudaError_t select_compact_setup() {
-  cudaError_t e = cudaFuncSetAttribute(select_compact_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
+  cudaError_t e = cudaFuncSetAttribute(copy_static_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStaticSmem);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(select_compact_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(select_compact_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
   if (e != cudaSuccess) return e;
@@ -1086,13 +1114,25 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   // many rows smaller clusters pay, because two CTAs per SM times the SM count is all that runs at once.
   const bool list = select && p.list && list_applies(p.E, p.k_q, p.row_stride);
   const bool sketch = list || (select && p.sketch && sketch_fits(p.E, p.row_stride));   // both read the row unstaged, if at all
-  // cluster size: slices of at least 2048 scores, at most 8 CTAs (the portable limit)
+  // Cluster size, at most 8 CTAs (the portable limit).
   int cs = 1;
-  // From a candidate list nothing but the gather scales with the cluster: a CTA takes up to 128 rows (one round of
-  // its 16 warps), and small launches leave room for the next launch's CTAs to run ahead (sagekv_set_select_overlap).
   const bool ahead = list && p.pdl == 2;
-  while (cs < kMaxCluster && (int64_t)cs * 2048 < p.E &&
-         (ahead ? (p.k_q + cs - 1) / cs > 128 : (!sketch || (int64_t)n_rows * cs * 2 <= 2 * (int64_t)n_sm))) cs <<= 1;
+  if (ahead) {
+    // From a candidate list nothing but the gather scales with the cluster: a CTA takes up to 128 rows (one round of
+    // its 16 warps), and small launches leave room for the next launch's CTAs to run ahead (sagekv_set_select_overlap).
+    while (cs < kMaxCluster && (int64_t)cs * 2048 < p.E && (p.k_q + cs - 1) / cs > 128) cs <<= 1;
+  } else if (sketch) {
+    while (cs < kMaxCluster && (int64_t)cs * 2048 < p.E && (int64_t)n_rows * cs * 2 <= 2 * (int64_t)n_sm) cs <<= 1;
+  } else {
+    // Slices of at most 16384 scores (one iteration of the passes, and two staged slices fit on an SM), as many CTAs as
+    // the prefilter wants thread maxima for k_q, and beyond that only what brings one CTA to every SM: more would not shorten
+    // the chain of block-wide steps that bounds short rows (us per launch with clusters of 8 / 4 / 2: 32 rows x
+    // 16251 14.9 / 11.8 / 12.6, 64 x 25236 with k_q = 1024 52.4 / 40.9 / 62.0, 128 x 6143 with k_q = 512 72.4 / 49.2 / 39.0,
+    // 128 x 59867 60.7 / 39.6 / 41.6, 32 x 130939 18.6 / 18.6 / 26.0).
+    while (cs < kMaxCluster && (int64_t)cs * 512 < p.E &&
+           ((int64_t)cs * 4 * 8 * kSelThreads < p.E || 2 * (int64_t)p.k_q > (int64_t)cs * kSelThreads || (int64_t)n_rows * cs * 2 <= n_sm))
+      cs <<= 1;
+  }
   int chunk = (p.E + cs - 1) / cs;
   chunk = (chunk + 3) & ~3;
   if (chunk < 4) chunk = 4;
@@ -1106,40 +1146,47 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   const bool resident = !sketch && select_smem_bytes(chunk, list_cap, cand_cap, share, true) <= (size_t)kSelSmemLimit;
   const size_t smem = select_smem_bytes(chunk, list_cap, cand_cap, share, resident);
 
-  // Without a selection (k_q = 0 or an empty eviction region) there are no row clusters: plain copy clusters
-  // move the sink, recent and last rows.  Otherwise the row clusters copy them along with the kept rows.
-  int copy_clusters = 0;
-  if (!select) {
-    const int static_items = p.B * p.H_kv * (p.S + p.R + 1);
-    copy_clusters = (static_items + cs * kSelWarps * 2 - 1) / (cs * kSelWarps * 2);
-    if (copy_clusters < 1) copy_clusters = 1;
-    const int cap = (n_sm + cs - 1) / cs;
-    if (copy_clusters > cap) copy_clusters = cap;
-  }
-
+  // Only launches that start from a candidate list are short enough to gain from early scheduling: the others
+  // pass over the row, and successors scheduled early take bandwidth and SM room from that.
+  SelectParams pl = p;
+  if (!list) pl.pdl = 0;
+  // The sink, recent and last rows: the row clusters copy them along with the kept rows as long as that is at most one
+  // row per warp.  More of them (the window is then a large share of the budget) would queue up behind the selection.  (us
+  // per launch along / beside, 4097 rows per head: 64 score rows of 25236 40.6 / 35.3, 32 of them 30.5 / 23.6.)
+  const int n_static = p.Kc != nullptr ? p.S + p.R + 1 : 0;
+  const bool beside = n_static > 0 && (!select || n_static > p.G * cs * kSelWarps);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n_rows + copy_clusters) * cs), 1, 1);
+  cudaLaunchAttribute attr[2];
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  if (beside) {
+    const int items = p.B * p.H_kv * ((n_static + 3) / 4), per_cta = kStaticThreads / 32 * kStaticStages;
+    int ctas = (items + per_cta - 1) / per_cta;
+    if (ctas > n_sm) ctas = n_sm;
+    cfg.gridDim = dim3((unsigned)ctas, 1, 1);
+    cfg.blockDim = dim3(kStaticThreads, 1, 1);
+    cfg.dynamicSmemBytes = kStaticSmem;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = pl.pdl ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, copy_static_kernel, pl, (int)!select);
+    if (e != cudaSuccess || !select) return e;
+  }
+  cfg.gridDim = dim3((unsigned)(n_rows * cs), 1, 1);
   cfg.blockDim = dim3(kSelThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  // Only launches that start from a candidate list are short enough to gain from early scheduling: the others
-  // pass over the row, and successors scheduled early take bandwidth and SM room from that.
-  SelectParams pl = p;
-  if (!list) pl.pdl = 0;
-  cfg.numAttrs = pl.pdl ? 2 : 1;
+  cfg.numAttrs = pl.pdl || beside ? 2 : 1;
   const int64_t sketch_off = try_fast && sketch && !list ? sketch_offset(p.E) : (int64_t)-1;
   const int64_t list_off = try_fast && list ? sketch_offset(p.E) : (int64_t)-1;
-  return ahead ? cudaLaunchKernelEx(&cfg, select_compact_kernel<true>, pl, n_rows, chunk, (int)resident, list_cap, cand_cap,
+  return ahead ? cudaLaunchKernelEx(&cfg, select_compact_kernel<true>, pl, (int)beside, chunk, (int)resident, list_cap, cand_cap,
                                     try_fast, sketch_off, list_off)
-               : cudaLaunchKernelEx(&cfg, select_compact_kernel<false>, pl, n_rows, chunk, (int)resident, list_cap, cand_cap,
+               : cudaLaunchKernelEx(&cfg, select_compact_kernel<false>, pl, (int)beside, chunk, (int)resident, list_cap, cand_cap,
                                     try_fast, sketch_off, list_off);
 }
 
