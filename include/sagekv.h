@@ -170,8 +170,9 @@ int sagekv_decode_attn(sagekv_ctx *ctx, const void *q, const void *k_new, const 
 /* How sagekv_decode_attn launches overlap with the kernel before them on the
  * stream.  Step 4 runs once per layer and per generated token, so at batch 1 the
  * launch-to-launch gap is a large share of its cost.  (The score launches are
- * always plain; sagekv_set_select_overlap covers select+compact.)
- *   0  (default) plain launch: starts when the previous kernel has finished.
+ * always as in mode 0; sagekv_set_select_overlap covers select+compact.)
+ *   0  (default) the kernel begins when the previous kernel has finished (only
+ *      its set-up may overlap that kernel's end), and releases nothing early.
  *   1  programmatic dependent launch: the kernel may be scheduled while its
  *      predecessor drains, and waits on the device for the predecessor to
  *      finish before it reads or writes anything.  Always safe.
@@ -203,7 +204,8 @@ int sagekv_set_decode_variant(sagekv_ctx *ctx, int variant);
  * and the pooled selection (Section 2, Steps 2 and 3), which run once per layer
  * after prefill and last a few microseconds each, so that with many layers queued
  * on a stream the gaps between them weigh as much as the work.
- *   0  (default) plain launch.
+ *   0  (default) begins when the previous kernel has finished (only its set-up
+ *      may overlap that kernel's end), and releases nothing early.
  *   1  programmatic dependent launch; the kernel waits on the device for its
  *      predecessor before it reads or writes anything a program can observe (it
  *      may ask for the candidate list to be brought into L2 earlier).  Always safe.
@@ -215,7 +217,7 @@ int sagekv_set_decode_variant(sagekv_ctx *ctx, int variant);
  *      for example the select call of another layer, when the score calls of all
  *      layers were queued first.
  * Launches that do not start from a candidate list (select hint modes 0 and 1)
- * pass over the score rows and are always plain, whatever the mode.
+ * pass over the score rows and are always as in mode 0, whatever the mode.
  * Errors: INVALID for a null context or a mode outside 0..2. */
 int sagekv_set_select_overlap(sagekv_ctx *ctx, int mode);
 

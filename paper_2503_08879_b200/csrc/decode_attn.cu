@@ -200,8 +200,8 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
   // the kernel directly before this one does not write this layer's cache.  The successor is released only
   // after the wait, so at most one kernel runs ahead of its dependency.
   if (p.pdl_mode < 2) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    wait_for_predecessor();
+    if (p.pdl_mode == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
   // ---- the warp that issues the copies: lane i takes requests i, i + 32, ... (two boxes per tile) ----
@@ -299,7 +299,7 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
 
   SAGEKV_STAMP(1);
   if (p.pdl_mode >= 2) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_predecessor();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
   SAGEKV_STAMP(2);
@@ -859,7 +859,7 @@ cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStre
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = p.pdl_mode > 0 ? 2 : 1;
+  cfg.numAttrs = 2;
   if (streamed) {
     const int heads = p.B * p.H_kv;
     cfg.gridDim = dim3((unsigned)(split > 1 ? heads * split : (heads + heads_per_cta - 1) / heads_per_cta), 1, 1);

@@ -148,8 +148,8 @@ decode_attn_tc_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
   cluster.barrier_arrive();                              // waited for just before the first store into a peer
 
   if (p.pdl_mode < 2) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    wait_for_predecessor();
+    if (p.pdl_mode == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
   // ---- the ninth warp: requests the copies, then issues the two products ----
@@ -272,7 +272,7 @@ decode_attn_tc_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
 
   SAGEKV_STAMP(1);
   if (p.pdl_mode >= 2) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_predecessor();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
   SAGEKV_STAMP(2);

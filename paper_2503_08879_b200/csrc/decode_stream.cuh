@@ -86,8 +86,8 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
   __syncwarp();
   if (split > 1) cluster.barrier_arrive();               // waited for before the first store into a peer: its barrier is set up
   if (p.pdl_mode < 2) {                                  // (see decode_attn_kernel: nothing is read or written before the wait, but for mode 2)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    wait_for_predecessor();
+    if (p.pdl_mode == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
   // the next tile to request: index rx in my range, tile rt of head rk of batch entry rb
@@ -133,7 +133,7 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
     }
 
   if (p.pdl_mode >= 2) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_predecessor();
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 

@@ -17,6 +17,7 @@ __global__ void __launch_bounds__(kScoreWarps * 32) score_logits_kernel(const Sc
   const int chunk = blockIdx.x, kvh = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, c = lane & 3;
+  wait_for_predecessor();
   if (chunk == 0 && p.sketch_off >= 0) {   // the rows' histograms are filled by atomic adds in the second pass
     for (int i = threadIdx.x; i < p.G * (kSketchBins + 4); i += kScoreWarps * 32) {
       const int h = i / (kSketchBins + 4);
@@ -119,6 +120,7 @@ constexpr int kFinalizeThreads = 256;
 __global__ void __launch_bounds__(kFinalizeThreads) score_finalize_kernel(const ScoreParams p, int per_slice) {
   const int row = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  wait_for_predecessor();
   float m = -INFINITY, l = 0.f;
   const float2 *part = p.partials + (int64_t)row * p.n_chunks;
   for (int i = threadIdx.x; i < p.n_chunks; i += kFinalizeThreads) {
@@ -171,6 +173,7 @@ constexpr int kSketchThreads = kSketchGroups;
 __global__ void __launch_bounds__(kSketchThreads) score_finalize_sketch_kernel(const ScoreParams p, int chunk) {
   const int row = blockIdx.y, slice = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  wait_for_predecessor();
   float m = -INFINITY, l = 0.f;
   const float2 *part = p.partials + (int64_t)row * p.n_chunks;
   for (int i = tid; i < p.n_chunks; i += kSketchThreads) {
@@ -246,15 +249,12 @@ cudaError_t launch_score(const ScoreParams &p_in, int n_sm, cudaStream_t stream)
   const bool list = p.list_k_q > 0 && list_applies(p.E, p.list_k_q, p.row_stride);
   p.sketch_off = !list && p.sketch && sketch_fits(p.E, p.row_stride) ? sketch_offset(p.E) : (int64_t)-1;
   dim3 grid(p.n_chunks, p.H_kv, p.B);
-  score_logits_kernel<<<grid, kScoreWarps * 32, 0, stream>>>(p);
-  cudaError_t err = cudaGetLastError();
+  cudaError_t err = launch_next(score_logits_kernel, grid, kScoreWarps * 32, 0, stream, 0, p);
   if (err != cudaSuccess) return err;
   if (list) return launch_score_finalize_candidates(p, stream);
   const int rows = p.B * p.H_q;
-  if (p.sketch_off >= 0) {
-    score_finalize_sketch_kernel<<<dim3(kSketchSlices, rows), kSketchThreads, 0, stream>>>(p, sketch_chunk(p.E));
-    return cudaGetLastError();
-  }
+  if (p.sketch_off >= 0)
+    return launch_next(score_finalize_sketch_kernel, dim3(kSketchSlices, rows), kSketchThreads, 0, stream, 0, p, sketch_chunk(p.E));
   int slices = (n_sm * 4 + rows - 1) / rows;
   const int max_slices = (p.E + 1023) / 1024;
   if (slices > max_slices) slices = max_slices;
@@ -262,8 +262,7 @@ cudaError_t launch_score(const ScoreParams &p_in, int n_sm, cudaStream_t stream)
   int per_slice = (p.E + slices - 1) / slices;
   per_slice = (per_slice + 3) & ~3;
   slices = (p.E + per_slice - 1) / per_slice;
-  score_finalize_kernel<<<dim3(slices, rows), kFinalizeThreads, 0, stream>>>(p, per_slice);
-  return cudaGetLastError();
+  return launch_next(score_finalize_kernel, dim3(slices, rows), kFinalizeThreads, 0, stream, 0, p, per_slice);
 }
 
 }  // namespace sagekv

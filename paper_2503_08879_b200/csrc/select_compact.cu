@@ -121,8 +121,7 @@ constexpr int kStaticSmem = (kStaticThreads / 32) * kStaticStages * 4 * 512;
 
 __global__ void __launch_bounds__(kStaticThreads, 8) copy_static_kernel(const SelectParams p, int alone) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  // (dependent launches: the selection that follows must find its inputs complete as soon as it starts)
-  if (p.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
+  wait_for_predecessor();                                // the selection that follows must find its inputs complete as soon as it starts
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per_head = p.S + p.R + 1, groups = (per_head + 3) >> 2, items = p.B * p.H_kv * groups;
@@ -733,16 +732,16 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   // write: selection and the first round of row loads run ahead of it, on the candidate-list path.
   // behind_static: the predecessor is this call's copy_static_kernel, which has found the inputs complete: nothing
   // here depends on it, but this kernel's end stands for the whole call's, so it waits before it ends.
-  bool waited = p.pdl == 0 || behind_static;
+  bool waited = behind_static != 0;
   if (p.pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (!waited && (p.pdl == 1 || list_off < 0)) {
-    if (list_off >= 0) {
+  if (!waited && (p.pdl < 2 || list_off < 0)) {
+    if (p.pdl && list_off >= 0) {
       const char *lines = reinterpret_cast<const char *>(p.scores + (int64_t)cid * p.row_stride + list_off);
       const int n_lines = (kListTagWords * 4 + cand_cap * 8 + 127) >> 7;
       const int mine = rank + (int)threadIdx.x * cs;
       if (mine < n_lines) asm volatile("prefetch.global.L2 [%0];" ::"l"(lines + (int64_t)mine * 128));
     }
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_predecessor();
     waited = true;
   }
   SAGEKV_STAMP(1);
@@ -843,14 +842,14 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
       SAGEKV_STAMP(6);
       idx_deferred = !waited && code == kFastDone;
       if (code == kFastGeneral) {                          // (a large group of equal scores at the cut)
-        if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
+        if (!waited) { wait_for_predecessor(); waited = true; }
         c.list = reinterpret_cast<int2 *>(c.scratch + kGeneralScratch);
         general_select(cluster, sh, p, c);
         code = kFastDone;
       }
       done = true;
     }
-    if (!done && !waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }   // the other paths write as they go
+    if (!done && !waited) { wait_for_predecessor(); waited = true; }   // the other paths write as they go
     if (!done && sketch_off >= 0 && tag0 == kSketchMagic && tag1 == (uint32_t)p.E)   // the same words in every CTA of the row
       code = resident ? fast_select<true, true>(cluster, sh, p, c, hint, false)
                       : fast_select<false, true>(cluster, sh, p, c, hint, false);
@@ -865,7 +864,7 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
     cluster.barrier_wait();
   }
   if (!done) {
-    if (!waited) { asm volatile("griddepcontrol.wait;" ::: "memory"); waited = true; }
+    if (!waited) { wait_for_predecessor(); waited = true; }
     c.list = reinterpret_cast<int2 *>(c.scratch + kGeneralScratch);
     general_select(cluster, sh, p, c);
   }
@@ -904,7 +903,7 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
       }
     }
     if (!waited) {                                         // the first write of this warp
-      asm volatile("griddepcontrol.wait;" ::: "memory");
+      wait_for_predecessor();
       waited = true;
     }
 #pragma unroll
@@ -922,7 +921,7 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
       sr += static_stride;
     }
   }
-  if (!waited || behind_static) asm volatile("griddepcontrol.wait;" ::: "memory");   // (not waited: a warp without a round of the loop)
+  if (!waited || behind_static) wait_for_predecessor();   // (not waited: a warp without a round of the loop)
   if (idx_deferred)                                        // every thread is here, and past the wait
     for (int i = tid; i < n_list_all; i += kSelThreads) {
       const int2 sp = c.list[i];
@@ -954,6 +953,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_finalize_candidates_kern
   cluster.barrier_arrive();   // completed in fast_candidates: every CTA of the cluster runs before anyone writes into a peer
   SAGEKV_TRACE_BEGIN
   SAGEKV_STAMP(0);
+  wait_for_predecessor();
   SelShared &sh = *reinterpret_cast<SelShared *>(smem_raw);
   float *staged = reinterpret_cast<float *>(smem_raw + sizeof(SelShared));
   SelCtx c;
@@ -1091,19 +1091,8 @@ cudaError_t launch_score_finalize_candidates(const ScoreParams &sp, cudaStream_t
   p.E = sp.E;
   p.k_q = sp.list_k_q;
   p.status = sp.status;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(rows * cs), 1, 1);
-  cfg.blockDim = dim3(kSelThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, score_finalize_candidates_kernel, sp, p, chunk, (int)resident, cand_cap, sketch_offset(sp.E));
+  return launch_next(score_finalize_candidates_kernel, dim3((unsigned)(rows * cs)), kSelThreads, smem, stream, cs, sp, p, chunk,
+                     (int)resident, cand_cap, sketch_offset(sp.E));
 }
 
 cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t stream) {
@@ -1146,8 +1135,8 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   const bool resident = !sketch && select_smem_bytes(chunk, list_cap, cand_cap, share, true) <= (size_t)kSelSmemLimit;
   const size_t smem = select_smem_bytes(chunk, list_cap, cand_cap, share, resident);
 
-  // Only launches that start from a candidate list are short enough to gain from early scheduling: the others
-  // pass over the row, and successors scheduled early take bandwidth and SM room from that.
+  // Only launches that start from a candidate list are short enough to gain from releasing their successor early: the
+  // others pass over the row, and successors scheduled early take bandwidth and SM room from that.
   SelectParams pl = p;
   if (!list) pl.pdl = 0;
   // The sink, recent and last rows: the row clusters copy them along with the kept rows as long as that is at most one
@@ -1155,39 +1144,17 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   // per launch along / beside, 4097 rows per head: 64 score rows of 25236 40.6 / 35.3, 32 of them 30.5 / 23.6.)
   const int n_static = p.Kc != nullptr ? p.S + p.R + 1 : 0;
   const bool beside = n_static > 0 && (!select || n_static > p.G * cs * kSelWarps);
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
-  cfg.stream = stream;
-  cfg.attrs = attr;
   if (beside) {
     const int items = p.B * p.H_kv * ((n_static + 3) / 4), per_cta = kStaticThreads / 32 * kStaticStages;
     int ctas = (items + per_cta - 1) / per_cta;
     if (ctas > n_sm) ctas = n_sm;
-    cfg.gridDim = dim3((unsigned)ctas, 1, 1);
-    cfg.blockDim = dim3(kStaticThreads, 1, 1);
-    cfg.dynamicSmemBytes = kStaticSmem;
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = pl.pdl ? 1 : 0;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, copy_static_kernel, pl, (int)!select);
+    const cudaError_t e = launch_next(copy_static_kernel, dim3((unsigned)ctas), kStaticThreads, kStaticSmem, stream, 0, pl, (int)!select);
     if (e != cudaSuccess || !select) return e;
   }
-  cfg.gridDim = dim3((unsigned)(n_rows * cs), 1, 1);
-  cfg.blockDim = dim3(kSelThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.numAttrs = pl.pdl || beside ? 2 : 1;
   const int64_t sketch_off = try_fast && sketch && !list ? sketch_offset(p.E) : (int64_t)-1;
   const int64_t list_off = try_fast && list ? sketch_offset(p.E) : (int64_t)-1;
-  return ahead ? cudaLaunchKernelEx(&cfg, select_compact_kernel<true>, pl, (int)beside, chunk, (int)resident, list_cap, cand_cap,
-                                    try_fast, sketch_off, list_off)
-               : cudaLaunchKernelEx(&cfg, select_compact_kernel<false>, pl, (int)beside, chunk, (int)resident, list_cap, cand_cap,
-                                    try_fast, sketch_off, list_off);
+  return launch_next(ahead ? select_compact_kernel<true> : select_compact_kernel<false>, dim3((unsigned)(n_rows * cs)), kSelThreads, smem,
+                     stream, cs, pl, (int)beside, chunk, (int)resident, list_cap, cand_cap, try_fast, sketch_off, list_off);
 }
 
 }  // namespace sagekv

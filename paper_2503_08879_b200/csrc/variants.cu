@@ -17,6 +17,7 @@ namespace sagekv {
 // kernel moves a few hundred rows), the products in double, one rounding to bf16 at the end.
 __global__ void __launch_bounds__(256) compact_window_rope_kernel(const WindowRopeParams p) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  wait_for_predecessor();
   const int L = p.S + p.R + 1;
   const int64_t n_rows = (int64_t)p.B * p.H_kv * L;
   const double log2_theta = log2((double)p.theta);
@@ -65,14 +66,14 @@ cudaError_t launch_compact_window_rope(const WindowRopeParams &p, int n_sm, cuda
   int64_t blocks = (n_rows + 7) / 8;
   if (blocks > 4 * (int64_t)n_sm) blocks = 4 * (int64_t)n_sm;
   if (blocks < 1) blocks = 1;
-  compact_window_rope_kernel<<<(unsigned)blocks, 256, 0, stream>>>(p);
-  return cudaGetLastError();
+  return launch_next(compact_window_rope_kernel, dim3((unsigned)blocks), 256, 0, stream, 0, p);
 }
 
 // ---- pooled scores -------------------------------------------------------------------------------------------
 // pooled[b, g, i] = sum over j < G of scores[b, g*G + j, i], added in head order in fp32.
 __global__ void __launch_bounds__(256) pool_scores_kernel(const float *scores, int64_t row_stride, float *pooled,
                                                           int64_t pooled_stride, int E, int G, int n_groups) {
+  wait_for_predecessor();
   const int n_vec = E >> 2;
   for (int g = blockIdx.y; g < n_groups; g += gridDim.y) {
     const float *src = scores + (int64_t)g * G * row_stride;
@@ -101,9 +102,8 @@ cudaError_t launch_pool_scores(const float *scores, int64_t row_stride, float *p
   const int want = (4 * n_sm + n_groups - 1) / n_groups;
   if (bx > want) bx = want;
   if (bx < 1) bx = 1;
-  pool_scores_kernel<<<dim3((unsigned)bx, (unsigned)(n_groups < 65535 ? n_groups : 65535)), 256, 0, stream>>>(
-      scores, row_stride, pooled, pooled_stride, E, G, n_groups);
-  return cudaGetLastError();
+  return launch_next(pool_scores_kernel, dim3((unsigned)bx, (unsigned)(n_groups < 65535 ? n_groups : 65535)), 256, 0, stream, 0,
+                     scores, row_stride, pooled, pooled_stride, E, G, n_groups);
 }
 
 // ---- Quest-style block summaries -----------------------------------------------------------------------------
@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(256) quest_build_kernel(const uint16_t *K, sag
                                                           int S, int E, int n_blocks, int H_kv) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int kvh = blockIdx.y, b = blockIdx.z;
+  wait_for_predecessor();
   const uint16_t *Kh = K + (int64_t)b * ks.batch_stride + (int64_t)kvh * ks.head_stride + (int64_t)S * ks.token_stride;
   for (int blk = blockIdx.x * 8 + warp; blk < n_blocks; blk += gridDim.x * 8) {
     float lo[8], hi[8];
@@ -155,8 +156,8 @@ cudaError_t launch_quest_build(const uint16_t *K, sagekv_strides ks, uint16_t *k
   int gx = (n_blocks + 7) / 8;
   const int want = (8 * n_sm + H_kv * B - 1) / (H_kv * B);
   if (gx > want) gx = want;
-  quest_build_kernel<<<dim3((unsigned)gx, (unsigned)H_kv, (unsigned)B), 256, 0, stream>>>(K, ks, kmin, kmax, S, E, n_blocks, H_kv);
-  return cudaGetLastError();
+  return launch_next(quest_build_kernel, dim3((unsigned)gx, (unsigned)H_kv, (unsigned)B), 256, 0, stream, 0, K, ks, kmin, kmax, S, E,
+                     n_blocks, H_kv);
 }
 
 // u[b, h, blk] = scale * sum_c max(q[b,h,c] * kmin[b, h/G, blk, c], q[b,h,c] * kmax[...]), fp32.  For finite summaries
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(256) quest_bounds_kernel(const uint16_t *q, co
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c = lane & 3;
   const int kvh = blockIdx.y, b = blockIdx.z;
   const int first = (blockIdx.x * 8 + warp) * 16;
+  wait_for_predecessor();
   if (first >= n_blocks) return;
   // lane (g, c) holds, of blocks first + g and first + g + 8, the 16-byte pieces at columns j*32 + c*8 of both summaries
   const int64_t base = ((int64_t)b * H_kv + kvh) * n_blocks;
@@ -246,9 +248,8 @@ __global__ void __launch_bounds__(256) quest_bounds_kernel(const uint16_t *q, co
 cudaError_t launch_quest_bounds(const uint16_t *q, const uint16_t *kmin, const uint16_t *kmax, float *u, int64_t u_stride,
                                 int n_blocks, int G, int H_q, int H_kv, int B, float scale, int n_sm, cudaStream_t stream) {
   if (n_blocks <= 0) return cudaSuccess;
-  quest_bounds_kernel<<<dim3((unsigned)((n_blocks + 127) / 128), (unsigned)H_kv, (unsigned)B), 256, 0, stream>>>(
-      q, kmin, kmax, u, u_stride, n_blocks, G, H_q, H_kv, scale);
-  return cudaGetLastError();
+  return launch_next(quest_bounds_kernel, dim3((unsigned)((n_blocks + 127) / 128), (unsigned)H_kv, (unsigned)B), 256, 0, stream, 0, q,
+                     kmin, kmax, u, u_stride, n_blocks, G, H_q, H_kv, scale);
 }
 
 }  // namespace sagekv
