@@ -172,7 +172,7 @@ int sagekv_decode_attn(sagekv_ctx *ctx, const void *q, const void *k_new, const 
  * launch-to-launch gap is a large share of its cost.  (The score launches are
  * always as in mode 0; sagekv_set_select_overlap covers select+compact.)
  *   0  (default) the kernel begins when the previous kernel has finished (only
- *      its set-up may overlap that kernel's end), and releases nothing early.
+ *      its set-up may overlap that kernel's end).
  *   1  programmatic dependent launch: the kernel may be scheduled while its
  *      predecessor drains, and waits on the device for the predecessor to
  *      finish before it reads or writes anything.  Always safe.

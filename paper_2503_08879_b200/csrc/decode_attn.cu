@@ -201,7 +201,7 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
   // after the wait, so at most one kernel runs ahead of its dependency.
   if (p.pdl_mode < 2) {
     wait_for_predecessor();
-    if (p.pdl_mode == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
   // ---- the warp that issues the copies: lane i takes requests i, i + 32, ... (two boxes per tile) ----

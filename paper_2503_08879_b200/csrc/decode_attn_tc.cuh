@@ -149,7 +149,7 @@ decode_attn_tc_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap 
 
   if (p.pdl_mode < 2) {
     wait_for_predecessor();
-    if (p.pdl_mode == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
   // ---- the ninth warp: requests the copies, then issues the two products ----

@@ -87,6 +87,8 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
   if (split > 1) cluster.barrier_arrive();               // waited for before the first store into a peer: its barrier is set up
   if (p.pdl_mode < 2) {                                  // (see decode_attn_kernel: nothing is read or written before the wait, but for mode 2)
     wait_for_predecessor();
+    // (mode 0: a successor waiting on the SMs from the start costs a launch that fills them, 256 heads x 2049 rows in four
+    // layers 177.6 -> 181.0 us)
     if (p.pdl_mode == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
