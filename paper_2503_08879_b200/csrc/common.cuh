@@ -15,7 +15,10 @@ constexpr float kLn2 = 0.6931471805599453f;
 
 // ---- score ---------------------------------------------------------------
 constexpr int kScoreWarps = 8;
-constexpr int kScoreTokPerWarp = 32;      // two 16-token mma tiles in flight per warp
+constexpr int kScoreTiles = 3;            // 16-token mma tiles a warp has in flight: 12 KB, so 192 KB per SM with two CTAs.  (us per
+                                          // score step, 8 KV heads x 130939 / 524155 tokens: three CTAs with two tiles per warp
+                                          // 51.6 / 197.5, this 49.7 / 188.4, four tiles 58.2 (spills), one tile 50.6)
+constexpr int kScoreTokPerWarp = kScoreTiles * 16;
 constexpr int kScoreChunk = kScoreWarps * kScoreTokPerWarp;   // tokens per CTA
 
 struct ScoreParams {

@@ -13,7 +13,7 @@
 
 namespace sagekv {
 
-__global__ void __launch_bounds__(kScoreWarps * 32) score_logits_kernel(const ScoreParams p) {
+__global__ void __launch_bounds__(kScoreWarps * 32, 2) score_logits_kernel(const ScoreParams p) {
   const int chunk = blockIdx.x, kvh = blockIdx.y, b = blockIdx.z;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int g = lane >> 2, c = lane & 3;
@@ -41,9 +41,9 @@ __global__ void __launch_bounds__(kScoreWarps * 32) score_logits_kernel(const Sc
   const int last = p.E - 1;
 
   // lane (g, c) holds, of token rows g and g+8 of each tile, the 16-byte pieces at columns j*32 + c*8
-  uint4 ka[2][4], kb[2][4];
+  uint4 ka[kScoreTiles][4], kb[kScoreTiles][4];
 #pragma unroll
-  for (int t = 0; t < 2; ++t) {
+  for (int t = 0; t < kScoreTiles; ++t) {
     const int r0 = min(tok_base + t * 16 + g, last);
     const int r1 = min(tok_base + t * 16 + g + 8, last);
     const char *pa = reinterpret_cast<const char *>(Kbase + (int64_t)r0 * p.ks.token_stride) + c * 16;
@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kScoreWarps * 32) score_logits_kernel(const Sc
   float *row1 = row0 + p.row_stride;
 
 #pragma unroll
-  for (int t = 0; t < 2; ++t) {
+  for (int t = 0; t < kScoreTiles; ++t) {
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -117,40 +117,60 @@ __global__ void __launch_bounds__(kScoreWarps * 32) score_logits_kernel(const Sc
 
 constexpr int kFinalizeThreads = 256;
 
-__global__ void __launch_bounds__(kFinalizeThreads) score_finalize_kernel(const ScoreParams p, int per_slice) {
-  const int row = blockIdx.y;
+// (max, 1 / sum) of a row from the (max, sum) pairs of the first pass's CTAs: the maximum first, then independent
+// exponentials instead of a chain of merges.  Every thread gets the result; sm holds kWarps pairs.
+template <int kWarps>
+__device__ __forceinline__ float2 row_max_and_inverse_sum(const float2 *part, int n, float2 (&sm)[kWarps]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  wait_for_predecessor();
   float m = -INFINITY, l = 0.f;
-  const float2 *part = p.partials + (int64_t)row * p.n_chunks;
-  for (int i = threadIdx.x; i < p.n_chunks; i += kFinalizeThreads) {
+  for (int i = threadIdx.x; i < n; i += kWarps * 32) {
     const float2 v = part[i];
     merge_ml(m, l, v.x, v.y);
   }
+  float wm = m;
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1)
-    merge_ml(m, l, __shfl_xor_sync(0xffffffffu, m, off), __shfl_xor_sync(0xffffffffu, l, off));
-  __shared__ float sm_m[kFinalizeThreads / 32], sm_l[kFinalizeThreads / 32];
-  if (lane == 0) { sm_m[warp] = m; sm_l[warp] = l; }
+  for (int off = 1; off < 32; off <<= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, off));
+  l = m == -INFINITY ? 0.f : l * fast_exp2(m - wm);
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+  if (lane == 0) sm[warp] = make_float2(wm, l);
   __syncthreads();
-  m = sm_m[0]; l = sm_l[0];
+  float2 w[kWarps];
 #pragma unroll
-  for (int w = 1; w < kFinalizeThreads / 32; ++w) merge_ml(m, l, sm_m[w], sm_l[w]);
-  const float inv = 1.f / l;
+  for (int i = 0; i < kWarps; ++i) w[i] = sm[i];
+  m = w[0].x;
+#pragma unroll
+  for (int i = 1; i < kWarps; ++i) m = fmaxf(m, w[i].x);
+  l = 0.f;
+#pragma unroll
+  for (int i = 0; i < kWarps; ++i) l += w[i].x == -INFINITY ? 0.f : w[i].y * fast_exp2(w[i].x - m);
+  return make_float2(m, 1.f / l);
+}
 
+// Eight 16-byte loads per thread and round are in flight before the first store (the row is read and written in place, so
+// the compiler would otherwise keep every load behind the previous store), the first round's ahead of the row's
+// maximum and sum, which they do not depend on.  Bound by latency, the logits being L2 hits: 32 rows of 130939 7.1 -> 6.9 us, the whole score step on 4096 tokens 6.4 -> 6.2.
+__global__ void __launch_bounds__(kFinalizeThreads) score_finalize_kernel(const ScoreParams p, int per_slice) {
+  const int row = blockIdx.y;
+  wait_for_predecessor();
   float *rowp = p.scores + (int64_t)row * p.row_stride;
   const int lo = blockIdx.x * per_slice;            // per_slice is a multiple of 4
   const int hi = min(p.E, lo + per_slice);
   if (!SAGEKV_OK_INDEX(p.status, row < p.B * p.H_q && lo >= 0 && (int64_t)hi <= p.row_stride)) return;
-  // eight 16-byte loads in flight per thread before the first store (the row is read and written in place,
-  // so the compiler would otherwise keep every load behind the previous store)
-  for (int i0 = lo + threadIdx.x * 4; i0 < hi; i0 += kFinalizeThreads * 4 * 8) {
-    float4 v[8];
+  float4 v[8];
+  auto load = [&](int i0) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int i = i0 + u * kFinalizeThreads * 4;
       if (i + 3 < hi) v[u] = *reinterpret_cast<const float4 *>(rowp + i);
     }
+  };
+  int i0 = lo + threadIdx.x * 4;
+  load(i0);
+  __shared__ float2 sm[kFinalizeThreads / 32];
+  const float2 ml = row_max_and_inverse_sum(p.partials + (int64_t)row * p.n_chunks, p.n_chunks, sm);
+  const float m = ml.x, inv = ml.y;
+  while (i0 < hi) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int i = i0 + u * kFinalizeThreads * 4;
@@ -162,6 +182,8 @@ __global__ void __launch_bounds__(kFinalizeThreads) score_finalize_kernel(const 
         for (int e = i; e < hi; ++e) rowp[e] = fast_exp2(rowp[e] - m) * inv;
       }
     }
+    i0 += kFinalizeThreads * 4 * 8;
+    if (i0 < hi) load(i0);
   }
 }
 
@@ -172,25 +194,8 @@ constexpr int kSketchThreads = kSketchGroups;
 
 __global__ void __launch_bounds__(kSketchThreads) score_finalize_sketch_kernel(const ScoreParams p, int chunk) {
   const int row = blockIdx.y, slice = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   wait_for_predecessor();
-  float m = -INFINITY, l = 0.f;
-  const float2 *part = p.partials + (int64_t)row * p.n_chunks;
-  for (int i = tid; i < p.n_chunks; i += kSketchThreads) {
-    const float2 v = part[i];
-    merge_ml(m, l, v.x, v.y);
-  }
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1)
-    merge_ml(m, l, __shfl_xor_sync(0xffffffffu, m, off), __shfl_xor_sync(0xffffffffu, l, off));
-  __shared__ float sm_m[kSketchThreads / 32], sm_l[kSketchThreads / 32];
-  if (lane == 0) { sm_m[warp] = m; sm_l[warp] = l; }
-  __syncthreads();
-  m = sm_m[0]; l = sm_l[0];
-#pragma unroll
-  for (int w = 1; w < kSketchThreads / 32; ++w) merge_ml(m, l, sm_m[w], sm_l[w]);
-  const float inv = 1.f / l;
-
   float *rowp = p.scores + (int64_t)row * p.row_stride;
   const int lo = slice * chunk;
   const int n_local = max(0, min(p.E - lo, chunk));
@@ -198,14 +203,21 @@ __global__ void __launch_bounds__(kSketchThreads) score_finalize_sketch_kernel(c
     return;
   const int n_vec = n_local >> 2;
   float *base = rowp + lo;
-  float fm = -INFINITY;
-  for (int v0 = 0; v0 < n_vec; v0 += 8 * kSketchThreads) {
-    float4 x[8];
+  float4 x[8];
+  auto load = [&](int v0) {
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int v = v0 + u * kSketchThreads + tid;
       if (v < n_vec) x[u] = *reinterpret_cast<const float4 *>(base + 4 * v);
     }
+  };
+  load(0);
+  __shared__ float2 sm[kSketchThreads / 32];
+  const float2 ml = row_max_and_inverse_sum(p.partials + (int64_t)row * p.n_chunks, p.n_chunks, sm);
+  const float m = ml.x, inv = ml.y;
+  float fm = -INFINITY;
+  for (int v0 = 0; v0 < n_vec; v0 += 8 * kSketchThreads) {
+    if (v0 > 0) load(v0);
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int v = v0 + u * kSketchThreads + tid;

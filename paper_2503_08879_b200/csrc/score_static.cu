@@ -12,7 +12,7 @@ using namespace sagekv;
 
 namespace {
 
-// (max, sum) pairs: one per score row and 256-token chunk of the eviction region.  256 KiB per GPU
+// (max, sum) pairs: one per score row and chunk of the eviction region, room for chunks of 256 tokens.  256 KiB per GPU
 // that loads the library, held until the process exits.
 constexpr int kStaticPartials = 32768;
 static __device__ __align__(256) float2 g_score_partials[kStaticPartials];
@@ -70,9 +70,10 @@ extern "C" int sagekv_score_static(const sagekv_shape *shape, const void *q_last
   if (!aligned16(q_last) || !aligned16(K) || !aligned16(scores) || ks.batch_stride % 8 || ks.head_stride % 8 ||
       ks.token_stride % 8 || scores_row_stride % 4)
     return SAGEKV_ERR_ALIGN;
+  // the fixed array bounds the problem: the interface promises room for one pair per row and 256 tokens
+  static_assert(kScoreChunk >= 256, "a CTA leaves at most one pair per row and 256 tokens");
+  if ((int64_t)shape->batch * shape->n_q_heads * ((E + 255) / 256) > kStaticPartials) return SAGEKV_ERR_TOO_LARGE;
   const int64_t n_chunks = (E + kScoreChunk - 1) / kScoreChunk;
-  // the fixed array bounds the problem: rows * chunks pairs must fit
-  if ((int64_t)shape->batch * shape->n_q_heads * n_chunks > kStaticPartials) return SAGEKV_ERR_TOO_LARGE;
   PerDevice *dev = nullptr;
   if (setup_current_device(&dev) != cudaSuccess) return SAGEKV_ERR_CUDA;
   ScoreParams p;
