@@ -39,6 +39,7 @@ constexpr int kSelThreads = 512;
 constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kMaxCluster = 8;
 constexpr int kMaxBins = 2048;
+constexpr int kRefineAbove = 48;                       // candidates at the cut that are ranked without a second histogram
 constexpr int kSelSmemLimit = 227 * 1024;             // the most a CTA can have on this part
 constexpr int kGeneralScratch = 4 * kMaxBins * 4;   // general path: three merged histograms and the local one
 
@@ -114,9 +115,10 @@ __device__ __forceinline__ void find_bin_from_top(const uint32_t *hist, int nb, 
 // several per warp: there they are launched ahead of the selection, which does not wait for them and leaves
 // the memory idle with its chain of barriers and scans, and run beside it on what two selection CTAs per SM leave of the
 // registers (8192) and of the shared memory.  A warp moves a row with 16 bytes per lane (K in lanes 0-15, V in lanes 16-31)
-// through a ring of its own in shared memory, 16 rows in flight, so 64 KB per SM.
+// through a ring of its own in shared memory, eight rows in flight, so 32 KB per SM: more queues up in front of the
+// selection's own loads (us per launch with 16 / 8 / 4 rows: 64 score rows of 25236 34.2 / 32.2 / 32.5).
 constexpr int kStaticThreads = 256;
-constexpr int kStaticStages = 4;          // of four rows
+constexpr int kStaticStages = 2;          // of four rows
 constexpr int kStaticSmem = (kStaticThreads / 32) * kStaticStages * 4 * 512;
 
 __global__ void __launch_bounds__(kStaticThreads, 8) copy_static_kernel(const SelectParams p, int alone) {
@@ -171,12 +173,18 @@ struct SelCtx {
   int list_cap;
   unsigned char *scratch;  // union: general-path histograms / fast-path candidate buffers
   int cand_cap;            // candidates per CTA and in total that the fast path can hold
+  uint32_t *masks;         // hits of the iterations of a slice that has several: [iteration][thread]
 };
 
 // Which 16-byte vectors of the CTA's slice a thread works on: vector (it*8 + u)*512 + tid for iteration it and
 // u = 0..7, so that a run of neighbouring scores is spread over as many threads as it has vectors (the bound of
 // step 1 is only tight when large scores do not share a thread).  (it, u, tid, element) order is position order.
-__device__ __forceinline__ int n_iterations(int n_vec) { return (n_vec + 8 * kSelThreads - 1) / (8 * kSelThreads); }
+__host__ __device__ __forceinline__ int n_iterations(int n_vec) { return (n_vec + 8 * kSelThreads - 1) / (8 * kSelThreads); }
+// shared memory for the hit masks of a slice of `chunk` scores
+__host__ __device__ __forceinline__ int mask_bytes(int chunk) {
+  const int n_it = n_iterations(chunk >> 2);
+  return n_it > 1 ? n_it * kSelThreads * 4 : 0;
+}
 
 // The eight vectors of iteration `it` of this thread, all loads issued before any use.  Missing ones read as
 // -inf, which is below every threshold and never a maximum.
@@ -390,6 +398,7 @@ __device__ int fast_candidates(cg::cluster_group &cluster, SelShared &sh, const 
   uint32_t mask = 0;                                     // of the last iteration (the only one when the slice is short)
   for (int it = 0; it < n_it; ++it) {
     mask = hit_mask(it);
+    if (n_it > 1) c.masks[it * kSelThreads + tid] = mask;
     uint32_t c_lo, c_hi;
     nibble_counts(mask, c_lo, c_hi);
     const uint32_t t_lo = __reduce_add_sync(0xffffffffu, c_lo), t_hi = __reduce_add_sync(0xffffffffu, c_hi);   // <= 128 per byte
@@ -413,7 +422,7 @@ __device__ int fast_candidates(cg::cluster_group &cluster, SelShared &sh, const 
   if (n_loc <= c.cand_cap) {
     int run_base = 0;                                    // hits of the iterations before this one
     for (int it = 0; it < n_it; ++it) {
-      if (n_it > 1) mask = hit_mask(it);
+      if (n_it > 1) mask = c.masks[it * kSelThreads + tid];    // (not read again: the slice is then not in shared memory)
       const uint32_t word = reinterpret_cast<const uint32_t *>(table)[it * 32 + lane];
       const uint32_t mine = byte_sum(word);
       uint32_t inc = mine;
@@ -494,11 +503,22 @@ __device__ int fast_candidates(cg::cluster_group &cluster, SelShared &sh, const 
     return kFastDone;
   }
   // every CTA takes a copy of all candidates, in CTA order: the list is sorted by position
-  for (int i = tid; i < M; i += kSelThreads) {
-    int r = 0;
+  for (int i0 = tid; i0 < M; i0 += 4 * kSelThreads) {      // four remote loads in flight
+    unsigned long long v[4];
 #pragma unroll
-    for (int q = 1; q < kMaxCluster; ++q) r += i >= start[q] ? 1 : 0;
-    cand_all[i] = cluster.map_shared_rank(cand_local, r)[i - start[r]];
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + u * kSelThreads;
+      if (i < M) {
+        int r = 0, first = 0;
+#pragma unroll
+        for (int q = 1; q < kMaxCluster; ++q)
+          if (i >= start[q]) { r = q; first = start[q]; }
+        v[u] = cluster.map_shared_rank(cand_local, r)[i - first];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * kSelThreads < M) cand_all[i0 + u * kSelThreads] = v[u];
   }
   __syncthreads();
   // This CTA is done with its peers' shared memory (the values it read are stored and past a barrier); the
@@ -531,13 +551,36 @@ __device__ int fast_decide(cg::cluster_group &cluster, SelShared &sh, const Sele
   __syncthreads();
   find_bin_from_top(sh.hist_fast, kSelThreads, p.k_q, sh);
   const uint32_t b1 = (uint32_t)sh.found[0];
-  const int r1 = sh.found[1];                            // the k_q-th largest is the r1-th largest inside b1
+  int r1 = sh.found[1];                                  // the k_q-th largest is the r1-th largest inside b1
+  // Many candidates in that bin (scores crowd towards the bound, the more so the larger k_q is): a second histogram over
+  // the next nine bits of their keys narrows the cut down, since ranking is quadratic.  (us per launch without / with, 32 rows
+  // x 524155 with k_q = 2015: 51.3 / 37.7)
+  const int shift3 = shift2 > 9 ? shift2 - 9 : 0;
+  const uint32_t base3 = (base2 + b1) << (shift2 - shift3);
+  const bool refine = shift2 > 0 && (int)sh.hist_fast[b1] > kRefineAbove;   // the same in every CTA
+  uint32_t b2 = 0u;
+  auto bin_of = [&](uint32_t key) { return min((key >> shift2) - base2, (uint32_t)kSelThreads - 1u); };
+  auto sub_bin_of = [&](uint32_t key) { return min((key >> shift3) - base3, (uint32_t)kSelThreads - 1u); };
+  if (refine) {
+    __syncthreads();                                     // every thread has read the count and found[]
+    sh.hist_fast[tid] = 0u;
+    __syncthreads();
+    for (int i = tid; i < M; i += kSelThreads) {
+      const uint32_t key = (uint32_t)(cand_all[i] >> 32);
+      if (bin_of(key) == b1) atomicAdd(&sh.hist_fast[sub_bin_of(key)], 1u);
+    }
+    __syncthreads();
+    find_bin_from_top(sh.hist_fast, kSelThreads, r1, sh);
+    b2 = (uint32_t)sh.found[0];
+    r1 = sh.found[1];
+  }
   SAGEKV_STAMP_AT(tr, 3);
   uint32_t *border = sh.gmax;                            // free: every peer is past step 2
   for (int i = tid; i < M; i += kSelThreads) {
-    const uint32_t bin = min((uint32_t)(cand_all[i] >> (32 + shift2)) - base2, (uint32_t)kSelThreads - 1u);
-    flag[i] = bin > b1 ? 1 : 0;
-    if (bin == b1) {
+    const uint32_t key = (uint32_t)(cand_all[i] >> 32), bin = bin_of(key);
+    const uint32_t sub = refine && bin == b1 ? sub_bin_of(key) : 0u;
+    flag[i] = bin > b1 || (bin == b1 && sub > b2) ? 1 : 0;
+    if (bin == b1 && sub == b2) {
       const int n = atomicAdd(&sh.n_border, 1);
       if (n < kSelThreads) border[n] = (uint32_t)i;
     }
@@ -749,7 +792,8 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   cluster.barrier_arrive();   // completed below: every CTA of the cluster runs before anyone writes into a peer
   SelShared &sh = *reinterpret_cast<SelShared *>(smem_raw);
   float *staged = reinterpret_cast<float *>(smem_raw + sizeof(SelShared));
-  unsigned char *after = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
+  unsigned char *masks = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
+  unsigned char *after = masks + mask_bytes(chunk);
   SelCtx c;
   c.cs = cs; c.rank = rank; c.row = cid; c.chunk = chunk;
   c.lo = rank * chunk;
@@ -758,6 +802,7 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   c.list_cap = list_cap;
   c.scratch = after;          // 16-byte aligned
   c.cand_cap = cand_cap;
+  c.masks = reinterpret_cast<uint32_t *>(masks);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = c.row / p.H_q, h = c.row - b * p.H_q;
@@ -962,8 +1007,10 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_finalize_candidates_kern
   c.n_local = max(0, min(p.E - c.lo, chunk));
   c.list = nullptr;
   c.list_cap = 0;
-  c.scratch = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
+  unsigned char *masks = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
+  c.scratch = masks + mask_bytes(chunk);
   c.cand_cap = cand_cap;
+  c.masks = reinterpret_cast<uint32_t *>(masks);
   sh.hist_fast[tid] = 0;
 
   // (max, sum) of the row from the first pass's partials
@@ -1066,11 +1113,14 @@ static size_t select_smem_bytes(int chunk, int list_cap, int cand_cap, int share
   const size_t general = (size_t)kGeneralScratch + (size_t)list_cap * sizeof(int2);
   if (scratch < general) scratch = general;
   scratch = (scratch + 15) & ~(size_t)15;
-  return sizeof(SelShared) + scratch + (resident ? (size_t)chunk * sizeof(float) : 0);
+  return sizeof(SelShared) + scratch + (size_t)mask_bytes(chunk) + (resident ? (size_t)chunk * sizeof(float) : 0);
 }
 
 cudaError_t select_compact_setup() {
   cudaError_t e = cudaFuncSetAttribute(copy_static_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kStaticSmem);
+  if (e != cudaSuccess) return e;
+  // (or an SM that has set aside less than two selection CTAs need keeps the second one waiting for its end)
+  e = cudaFuncSetAttribute(copy_static_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(select_compact_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
   if (e != cudaSuccess) return e;
@@ -1105,14 +1155,18 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   const bool sketch = list || (select && p.sketch && sketch_fits(p.E, p.row_stride));   // both read the row unstaged, if at all
   // Cluster size, at most 8 CTAs (the portable limit).
   int cs = 1;
-  const bool ahead = list && p.pdl == 2;
+  const int n_static = p.Kc != nullptr ? p.S + p.R + 1 : 0;   // sink, recent and last rows per KV head
+  bool ahead = list && p.pdl == 2;
   if (ahead) {
     // From a candidate list nothing but the gather scales with the cluster: a CTA takes up to 128 rows (one round of
     // its 16 warps), and small launches leave room for the next launch's CTAs to run ahead (sagekv_set_select_overlap).
     while (cs < kMaxCluster && (int64_t)cs * 2048 < p.E && (p.k_q + cs - 1) / cs > 128) cs <<= 1;
-  } else if (sketch) {
+    ahead = n_static <= p.G * cs * kSelWarps;            // (more static rows are copied beside: see below)
+    if (!ahead) cs = 1;
+  }
+  if (!ahead && sketch) {
     while (cs < kMaxCluster && (int64_t)cs * 2048 < p.E && (int64_t)n_rows * cs * 2 <= 2 * (int64_t)n_sm) cs <<= 1;
-  } else {
+  } else if (!ahead) {
     // Slices of at most 16384 scores (one iteration of the passes, and two staged slices fit on an SM), as many CTAs as
     // the prefilter wants thread maxima for k_q, and beyond that only what brings one CTA to every SM: more would not shorten
     // the chain of block-wide steps that bounds short rows (us per launch with clusters of 8 / 4 / 2: 32 rows x
@@ -1135,15 +1189,14 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   const bool resident = !sketch && select_smem_bytes(chunk, list_cap, cand_cap, share, true) <= (size_t)kSelSmemLimit;
   const size_t smem = select_smem_bytes(chunk, list_cap, cand_cap, share, resident);
 
-  // Only launches that start from a candidate list are short enough to gain from releasing their successor early: the
-  // others pass over the row, and successors scheduled early take bandwidth and SM room from that.
-  SelectParams pl = p;
-  if (!list) pl.pdl = 0;
   // The sink, recent and last rows: the row clusters copy them along with the kept rows as long as that is at most one
   // row per warp.  More of them (the window is then a large share of the budget) would queue up behind the selection.  (us
-  // per launch along / beside, 4097 rows per head: 64 score rows of 25236 40.6 / 35.3, 32 of them 30.5 / 23.6.)
-  const int n_static = p.Kc != nullptr ? p.S + p.R + 1 : 0;
+  // per launch along / beside, 4097 rows per head: 64 score rows of 25236 40.6 / 32.2, 32 of them 30.5 / 23.7.)
   const bool beside = n_static > 0 && (!select || n_static > p.G * cs * kSelWarps);
+  // Only launches that start from a candidate list, and copy all rows themselves, are short enough to gain from releasing
+  // their successor early: successors scheduled early take bandwidth and SM room from the others.
+  SelectParams pl = p;
+  if (!list || beside) pl.pdl = 0;
   if (beside) {
     const int items = p.B * p.H_kv * ((n_static + 3) / 4), per_cta = kStaticThreads / 32 * kStaticStages;
     int ctas = (items + per_cta - 1) / per_cta;
