@@ -10,7 +10,7 @@
 //
 // What bounds it: HBM where all SMs are full (256 heads x 2049 rows: 42.8 us per launch, 6.3 TB/s; decode_attn_kernel,
 // whose whole-SM CTAs load, compute and merge one after another, took 84.8), else the tiles a warp takes one after
-// another at 0.6 us each, three in flight per warp (8 heads x 8193 rows over 16 CTAs per head: 9.4 us against 11.0).
+// another at 0.6 us each, three in flight per warp (8 heads x 8193 rows over 16 CTAs per head: 8.7 us against 11.0).
 // Two CTAs per SM, so that a launch's copies start while its predecessor still computes and merges; 4 warps x 3 stages,
 // 8 warps with single slots and a first product one tile ahead measured the same within 3 %.
 #pragma once
@@ -134,13 +134,20 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
       if (first < z) my_win += (z - 1 - first) / kStWarps + 1;
     }
 
+  // Mode 2: when the successor may start.  Its copies compete with this launch's own as long as there are any to request, and
+  // later, while this launch merges, the memory would be idle: a part of more than twice the ring releases it with its
+  // last requests.  (us per launch at once / so: 8 heads x 8193 rows 9.18 / 8.74, 16 x 4097 9.43 / 8.71, 24 x 8193
+  // 17.95 / 17.22; but 17 tiles per CTA, 8 x 4097, 5.69 / 5.91, and whole heads, 256 x 2049, 42.1 / 42.7)
+  const bool release_late = split > 1 && n_tiles > 2 * kStWarps * kStStages * split;
   if (p.pdl_mode >= 2) {
     wait_for_predecessor();
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!release_late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
+  const uint32_t ring_magic = 0xffffffffu / (uint32_t)max(p.ring_len, 1);   // (no division behind the wait)
   bool timed_out = false;
   int stage = 0, step = 0, my_ticket = -1, win_row = -1; // ring stage of my next tile; step counter; the replaced row of the window
+  if (my_win > 0) asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(step) : "l"(p.d_step));   // (ahead of the query's loads)
   uint32_t phase = 0;
   int x = warp;                                          // my next tile, as an index into the CTA's range
   int b = first_head / p.H_kv, kvh = first_head - b * p.H_kv;
@@ -164,12 +171,13 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
     if (my_win > 0) {
       new_row = ld_v4((lane < 16 ? p.k_new : p.v_new) + ((int64_t)b * p.H_kv + kvh) * kHeadDim + (lane & 15) * 8);
       if (win_row < 0) {
-        asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(step) : "l"(p.d_step));
         // a ticket per window tile, taken once the counter has been read (the increment depends on the value: see decode_attn_kernel)
         if (lane == 0)
           asm volatile("{ .reg .b32 inc; shr.u32 inc, %2, 31; add.u32 inc, inc, %3; atom.add.relaxed.gpu.global.s32 %0, [%1], inc; }"
                        : "=r"(my_ticket) : "l"(p.tickets + heads), "r"(step), "r"(my_win) : "memory");
-        win_row = win_lo + (int)((uint32_t)step % (uint32_t)p.ring_len);
+        uint32_t r = (uint32_t)step - __umulhi((uint32_t)step, ring_magic) * (uint32_t)p.ring_len;
+        while (r >= (uint32_t)p.ring_len) r -= (uint32_t)p.ring_len;
+        win_row = win_lo + (int)r;
       }
     }
     const int patch_x = win_row >= 0 ? head_x0 + (win_row >> 4) : -1;
@@ -246,6 +254,7 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
       __syncwarp();                                      // every lane has its fragments: the stage may be refilled
       if (patch) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       request(stage);
+      if (release_late && rx >= n && p.pdl_mode >= 2) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
       if (++stage == kStStages) { stage = 0; phase ^= 1u; }
     }
 
