@@ -742,6 +742,7 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int
   int nc = (n_tiles + c * kDecodeMaxTiles - 1) / (c * kDecodeMaxTiles);          // the fewest clusters per head
   float best = 0.f;
   int best_waves = 1;
+  bool apart = false;                                    // two launches' clusters do not fit on the device together
   if (dev != nullptr && heads > 0) {
     int best_c = c, best_nc = nc;
     // up to kDecodeExtraClusters more clusters per head than needed: beyond one cluster the results are merged
@@ -761,7 +762,10 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int
         const float one = 2.97f + 0.0445f * (float)per * (2 * heads * n_try <= cap ? 1.f : 2.f) + 0.084f * (float)late +
                           (n_try > 1 ? 3.4f : 0.f);
         const float cost = (float)waves * one;
-        if (best == 0.f || cost < best) { best = cost; best_c = cand; best_nc = n_try; best_waves = waves; }
+        if (best == 0.f || cost < best) {
+          best = cost; best_c = cand; best_nc = n_try; best_waves = waves;
+          apart = 2 * heads * n_try > cap;
+        }
       }
     }
     c = best_c;
@@ -776,13 +780,16 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int
   *smem_bytes = (int)decode_smem_bytes(per_cta);
   // without overlap: 3.9 + 0.14 per tile (the copies are issued on the critical path: L = 257 .. 4097, 1 to 16 heads)
   if (best > 0.f && !overlap) best = (float)best_waves * (3.9f + 0.14f * (float)per_cta + (nc > 1 ? 3.4f : 0.f));
+  // (against the streamed launch: 16 / 24 / 32 heads x 2049 rows 5.9 / 7.7 / 8.5)
+  if (best > 0.f && overlap && apart) best += 0.027f * (float)(best_waves * per_cta);
   return best > 0.f ? with_traffic(best, heads, L) : 0.f;
 }
 
 // The best launch of decode_stream_kernel: CTAs per head, heads per CTA, and its cost in us (0: none).  Measured over
-// 1 to 600 heads and L = 257 .. 8193: 2.4 plus 0.6 per tile of a warp (the ring's three tiles per warp in flight against
-// the latency of a copy); 1.7 more when the launches do not overlap; up to 1.5 more when two launches' CTAs do
-// not fit on the device together; 0.8 per further head of a CTA; a second wave costs a whole time again.
+// 1 to 600 heads and L = 257 .. 8193: 2 plus 0.025 per CTA of a cluster plus 0.6 per tile of a warp (the ring's three tiles
+// per warp in flight against the latency of a copy); 1.9 more when the launches do not overlap; up to 1.5 more when two
+// launches' CTAs do not fit on the device together (24 heads x 2049 rows over 8 CTAs each 6.7 against 7.7 whole); 0.8 per
+// further head of a CTA; a second wave costs a whole time again.
 static float stream_geometry(int L, int heads, const DeviceInfo &dev, bool overlap, int *split, int *per_cta) {
   const int n_tiles = (L + 15) / 16;
   if ((int64_t)n_tiles * heads > (int64_t)1 << 30) return 0.f;
@@ -794,10 +801,10 @@ static float stream_geometry(int L, int heads, const DeviceInfo &dev, bool overl
     const int ctas = s == 1 ? (heads + per - 1) / per : heads * s;
     const int waves = (ctas + cap - 1) / cap;
     const int rounds = (per * ((n_tiles + s - 1) / s) + kStWarps - 1) / kStWarps;
-    float one = 2.4f + 0.6f * (float)rounds + 0.8f * (float)(per - 1);
-    if (!overlap) one += 1.7f;
+    float one = 2.f + 0.025f * (float)s + 0.6f * (float)rounds + 0.8f * (float)(per - 1);
+    if (!overlap) one += 1.9f;
     float cost = with_traffic((float)waves * one, heads, L);
-    if (2 * ctas > cap) cost += 0.5f + (float)(2 * (ctas < cap ? ctas : cap) - cap) / (float)cap;
+    if (2 * ctas > cap) cost += 0.3f + 1.2f * (float)(2 * (ctas < cap ? ctas : cap) - cap) / (float)cap;
     if (best == 0.f || cost < best) { best = cost; *split = s; *per_cta = per; }
   }
   return best;
