@@ -167,7 +167,8 @@ cudaError_t launch_quest_build(const uint16_t *K, sagekv_strides ks, uint16_t *k
 // to 8) as the columns, and because a dot product does not care in which order its terms are added, the fragments are
 // filled from plain 16-byte loads with the summaries and the query in the same column order.
 // Bound by memory: 33.5 MB of summaries (8 KV heads x 8183 blocks) take 19.1 us with one product, one maximum and one
-// addition per head and element, 7.7 on the tensor cores.
+// addition per head and element, 8.2 on the tensor cores in CTAs of eight warps (two of them per SM) and 6.8 in CTAs of four
+// (five per SM: the last wave is shorter).
 __device__ __forceinline__ float bf16_at(const uint16_t *p) { return __uint_as_float((uint32_t)*p << 16); }
 
 // a <= b for all eight pairs (false for NaN)
@@ -180,11 +181,13 @@ __device__ __forceinline__ bool le_bf16x8(uint4 a, uint4 b) {
   return (le(a.x, b.x) & le(a.y, b.y) & le(a.z, b.z) & le(a.w, b.w)) == 0xffffffffu;
 }
 
-__global__ void __launch_bounds__(256) quest_bounds_kernel(const uint16_t *q, const uint16_t *kmin, const uint16_t *kmax, float *u,
+constexpr int kBoundsWarps = 4;
+
+__global__ void __launch_bounds__(kBoundsWarps * 32, 5) quest_bounds_kernel(const uint16_t *q, const uint16_t *kmin, const uint16_t *kmax, float *u,
                                                            int64_t u_stride, int n_blocks, int G, int H_q, int H_kv, float scale) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, c = lane & 3;
   const int kvh = blockIdx.y, b = blockIdx.z;
-  const int first = (blockIdx.x * 8 + warp) * 16;
+  const int first = (blockIdx.x * kBoundsWarps + warp) * 16;
   wait_for_predecessor();
   if (first >= n_blocks) return;
   // lane (g, c) holds, of blocks first + g and first + g + 8, the 16-byte pieces at columns j*32 + c*8 of both summaries
@@ -248,8 +251,9 @@ __global__ void __launch_bounds__(256) quest_bounds_kernel(const uint16_t *q, co
 cudaError_t launch_quest_bounds(const uint16_t *q, const uint16_t *kmin, const uint16_t *kmax, float *u, int64_t u_stride,
                                 int n_blocks, int G, int H_q, int H_kv, int B, float scale, int n_sm, cudaStream_t stream) {
   if (n_blocks <= 0) return cudaSuccess;
-  return launch_next(quest_bounds_kernel, dim3((unsigned)((n_blocks + 127) / 128), (unsigned)H_kv, (unsigned)B), 256, 0, stream, 0, q,
-                     kmin, kmax, u, u_stride, n_blocks, G, H_q, H_kv, scale);
+  const int per_cta = kBoundsWarps * 16;
+  return launch_next(quest_bounds_kernel, dim3((unsigned)((n_blocks + per_cta - 1) / per_cta), (unsigned)H_kv, (unsigned)B),
+                     kBoundsWarps * 32, 0, stream, 0, q, kmin, kmax, u, u_stride, n_blocks, G, H_q, H_kv, scale);
 }
 
 }  // namespace sagekv
