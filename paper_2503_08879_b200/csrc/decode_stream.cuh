@@ -69,6 +69,8 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
     first_tile = 0;
     n = min(per_cta, heads - first_head) * n_tiles;
   }
+  SAGEKV_TRACE_BEGIN
+  SAGEKV_STAMP(0);
   const int cols_log = 7 - (31 - __clz(split)), cols = 1 << cols_log;   // columns each CTA of a cluster finishes: 128 / split
 
   const uint32_t ring = smem_u32(&sh.ring[warp][0][0]), bars = smem_u32(&sh.bar[warp][0]), inbox_bar = smem_u32(&sh.inbox_bar);
@@ -139,12 +141,14 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
   // last requests.  (us per launch at once / so: 8 heads x 8193 rows 9.18 / 8.74, 16 x 4097 9.43 / 8.71, 24 x 8193
   // 17.95 / 17.22; but 17 tiles per CTA, 8 x 4097, 5.69 / 5.91, and whole heads, 256 x 2049, 42.1 / 42.7)
   const bool release_late = split > 1 && n_tiles > 2 * kStWarps * kStStages * split;
+  SAGEKV_STAMP(1);
   if (p.pdl_mode >= 2) {
     wait_for_predecessor();
     if (!release_late) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
   const uint32_t ring_magic = 0xffffffffu / (uint32_t)max(p.ring_len, 1);   // (no division behind the wait)
+  SAGEKV_STAMP(2);
   bool timed_out = false;
   int stage = 0, step = 0, my_ticket = -1, win_row = -1; // ring stage of my next tile; step counter; the replaced row of the window
   if (my_win > 0) asm volatile("ld.volatile.global.s32 %0, [%1];" : "=r"(step) : "l"(p.d_step));   // (ahead of the query's loads)
@@ -190,6 +194,7 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
     for (; x < x_end; x += kStWarps) {
       const uint32_t tb = ring + (uint32_t)(stage * kStStageBytes);
       if (!mbar_wait(bars + 8u * stage, phase)) timed_out = true;
+      if (x == 0) SAGEKV_STAMP(3);
       const bool patch = x == patch_x;                   // the staged copy of the replaced row is stale
       if (patch) {
         const uint32_t dst = tb + (lane < 16 ? 0u : (uint32_t)kSlotBytes) + tile_offset(win_row & 15, lane & 15);
@@ -258,6 +263,7 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
       if (++stage == kStStages) { stage = 0; phase ^= 1u; }
     }
 
+    SAGEKV_STAMP_AFTER(4, acc[0][0] + acc[7][3]);
     // ---- the head (or my part of it) is done: merge the four warps ----
 #pragma unroll
     for (int o = 4; o < 32; o <<= 1) {
@@ -278,6 +284,7 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
     }
     if (split > 1) cluster.barrier_wait();
     __syncthreads();
+    SAGEKV_STAMP(5);
     const int64_t row0 = (int64_t)b * p.H_q + kvh * p.G;   // the head's first row of out and lse
     for (int item = tid; item < p.G * (kHeadDim / 4); item += kStThreads) {
       const int h = item >> 5, col = (item & 31) * 4;
@@ -315,9 +322,11 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
         }
       }
     }
+    SAGEKV_STAMP(6);
     if (split > 1) {
       // ---- finish my columns from the inbox, two per thread ----
       if (!mbar_wait(inbox_bar, 0u)) timed_out = true;
+      SAGEKV_STAMP(7);
       for (int item = tid; item < (p.G << cols_log) >> 1; item += kStThreads) {
         const int h = item >> (cols_log - 1), lc = (item & ((cols >> 1) - 1)) * 2, col = rank * cols + lc;
         float2 ml[kStMaxCluster], v[kStMaxCluster];
@@ -344,11 +353,17 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
     }
     if (++kvh == p.H_kv) { kvh = 0; ++b; }
   }
+#if defined(SAGEKV_TRACE)
+  if (split == 1) trace_t[7] = trace_t[6];
+#endif
+  SAGEKV_STAMP(8);
   if (timed_out) atomicOr(p.status, kStatusWaitTimeout);
   if (my_win > 0 && lane == 0 && my_ticket + my_win == heads * (n_tiles - (win_lo >> 4))) {   // every reader has read the counter
     p.tickets[heads] = 0;
     *p.d_step = step + 1;
   }
+  SAGEKV_STAMP(9);
+  SAGEKV_TRACE_END(p.out);
 }
 
 }  // namespace sagekv

@@ -23,8 +23,13 @@ NAMES = ["CTA starts", "copies issued", "dependency wait over", "K landed", "max
          "second product done", "results sent", "inbox full", "CTA ends"]
 
 
-def report(buf_reader, names, ctas_of, run, label):
-    """Records one run and prints the phases; ctas_of(first record) = CTAs per launch."""
+# the streamed kernel (many heads, long caches); a CTA with several whole heads shows its last one
+STREAM_NAMES = ["CTA starts", "copies issued", "dependency wait over", "first tile landed", "last tile done", "results in shared memory",
+                "results sent", "inbox full", "outputs written", "CTA ends"]
+
+
+def report(buf_reader, names, run, label, heads=1):
+    """Records one run and prints the phases; heads: KV heads of a decode launch."""
     import torch
     buf = np.zeros((1 << 15, 12), dtype=np.uint64)
     n = C.c_uint(0)
@@ -36,7 +41,9 @@ def report(buf_reader, names, ctas_of, run, label):
     t = buf[: min(n.value, 1 << 15)].astype(np.int64)
     grid = t[:, 11] & 0xffffffff
     tags = t[:, 11] >> 32                          # which buffer the launch wrote: one value per layer
-    ctas = ctas_of(np.concatenate([t[0, :11], grid[:1]]))
+    ctas = int(grid[0])
+    if names is NAMES and ctas > 1 and not (t[:, 10] & 0xffffffff).any() and heads > 1:
+        names = STREAM_NAMES                       # (its launches are one-dimensional)
     groups = []                                    # launches may overlap in time: told apart by tag, then by start
     for tag in np.unique(tags):
         r = t[tags == tag]
@@ -103,7 +110,7 @@ def trace_select(argv):
         g.replay()
         return rounds * n_layers
 
-    report(B.lib.sagekv_trace_read_select, SELECT_NAMES, lambda r: int(r[11]), run,
+    report(B.lib.sagekv_trace_read_select, SELECT_NAMES, run,
            "%s select+compact, hint mode 2, overlap mode %d, %d layers" % (name, overlap, n_layers))
     sk.close()
 
@@ -148,8 +155,9 @@ def main(argv):
         g.replay()
         return steps * n_layers
 
-    report(B.lib.sagekv_trace_read, NAMES, lambda r: int(r[11]) * w.n_kv_heads * w.batch, run,
-           "%s decode, overlap mode %d, %d layers (cluster size %s)" % (name, overlap, n_layers, "= CTAs / (KV heads x batch)"))
+    report(B.lib.sagekv_trace_read, NAMES, run,
+           "%s decode, overlap mode %d, %d layers (cluster size %s)" % (name, overlap, n_layers, "= CTAs / (KV heads x batch)"),
+           heads=w.n_kv_heads * w.batch)
     sk.close()
 
 
