@@ -117,6 +117,7 @@ __device__ __forceinline__ void find_bin_from_top(const uint32_t *hist, int nb, 
 // registers (8192) and of the shared memory.  A warp moves a row with 16 bytes per lane (K in lanes 0-15, V in lanes 16-31)
 // through a ring of its own in shared memory, eight rows in flight, so 32 KB per SM: more queues up in front of the
 // selection's own loads (us per launch with 16 / 8 / 4 rows: 64 score rows of 25236 34.2 / 32.2 / 32.5).
+constexpr int kStaticPerWarp = 2;         // rows a warp of the row clusters copies along at most
 constexpr int kStaticThreads = 256;
 constexpr int kStaticStages = 2;          // of four rows
 constexpr int kStaticSmem = (kStaticThreads / 32) * kStaticStages * 4 * 512;
@@ -1176,7 +1177,7 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
     // From a candidate list nothing but the gather scales with the cluster: a CTA takes up to 128 rows (one round of
     // its 16 warps), and small launches leave room for the next launch's CTAs to run ahead (sagekv_set_select_overlap).
     while (cs < kMaxCluster && (int64_t)cs * 2048 < p.E && (p.k_q + cs - 1) / cs > 128) cs <<= 1;
-    ahead = n_static <= p.G * cs * kSelWarps;            // (more static rows are copied beside: see below)
+    ahead = n_static <= kStaticPerWarp * p.G * cs * kSelWarps;            // (more static rows are copied beside: see below)
     if (!ahead) cs = 1;
   }
   if (!ahead && sketch) {
@@ -1204,10 +1205,13 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   const bool resident = !sketch && select_smem_bytes(chunk, list_cap, cand_cap, share, true) <= (size_t)kSelSmemLimit;
   const size_t smem = select_smem_bytes(chunk, list_cap, cand_cap, share, resident);
 
-  // The sink, recent and last rows: the row clusters copy them along with the kept rows as long as that is at most one
-  // row per warp.  More of them (the window is then a large share of the budget) would queue up behind the selection.  (us
-  // per launch along / beside, 4097 rows per head: 64 score rows of 25236 40.6 / 32.2, 32 of them 30.5 / 23.7.)
-  const bool beside = n_static > 0 && (!select || n_static > p.G * cs * kSelWarps);
+  // The sink, recent and last rows: the row clusters copy them along with the kept rows as long as that is at most
+  // kStaticPerWarp rows per warp.  More of them (the window is then a large share of the budget) would queue up behind the
+  // selection; fewer are not worth a launch, nor the early start that a launch from candidate lists has without it.  (us per
+  // launch along / beside: 64 score rows of 25236, 4097 rows per head, 40.6 / 32.2, 32 of them 30.5 / 23.7; 16 pooled rows of
+  // 59862, 138 rows, 23.3 / 25.2; from candidate lists of 131072 tokens, 133 rows 4.5 / 6.6, 505 rows 5.8 / 7.4, 1005 rows,
+  // four per warp, 7.4 / 7.8, but 69.2 / 67.6 with the score launch in front.)
+  const bool beside = n_static > 0 && (!select || n_static > kStaticPerWarp * p.G * cs * kSelWarps);
   // Only launches that start from a candidate list, and copy all rows themselves, are short enough to gain from releasing
   // their successor early: successors scheduled early take bandwidth and SM room from the others.
   SelectParams pl = p;

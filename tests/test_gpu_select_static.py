@@ -1,4 +1,4 @@
-"""select+compact where the sink, recent and last rows are many: from one row per warp of the head's clusters on (both sides
+"""select+compact where the sink, recent and last rows are many: from two rows per warp of the head's clusters on (both sides
 of that line) a kernel of their own copies them beside the selection.  Every hint and overlap mode, several layers back to
 back, row strides beyond 128 elements; and the shapes of the score row at which the cluster size changes.  Bit-exact."""
 
@@ -55,7 +55,8 @@ def run(B, Bt, Hkv, G, E, k_q, S, R, hint=0, overlap=0, pad=0, layers=3):
 
 @pytest.mark.parametrize("Bt,Hkv,G,E,k_q,S,R,pad", [
     (1, 1, 1, 3000, 40, 40, 87, 0),      # 128 rows over a cluster of 8 x 16 warps: one per warp
-    (1, 1, 1, 3000, 40, 41, 87, 8),      # 129: beside
+    (1, 1, 1, 3000, 40, 41, 214, 0),     # 256: two per warp
+    (1, 1, 1, 3000, 40, 41, 215, 8),     # 257: beside
     (2, 4, 2, 5000, 300, 512, 900, 0),
     (1, 2, 4, 2001, 7, 0, 1500, 16),     # no sink
     (1, 2, 4, 2001, 7, 1500, 0, 0),      # no recent rows
