@@ -181,10 +181,11 @@ struct SelCtx {
 // u = 0..7, so that a run of neighbouring scores is spread over as many threads as it has vectors (the bound of
 // step 1 is only tight when large scores do not share a thread).  (it, u, tid, element) order is position order.
 __host__ __device__ __forceinline__ int n_iterations(int n_vec) { return (n_vec + 8 * kSelThreads - 1) / (8 * kSelThreads); }
-// shared memory for the hit masks of a slice of `chunk` scores
-__host__ __device__ __forceinline__ int mask_bytes(int chunk) {
+// Shared memory for the hit masks of a slice of `chunk` scores: the prefilter's alone.  It takes slices of at most 16
+// iterations (32 KB of masks); a longer slice goes the general way, whose shared memory must not grow with it.
+__host__ __device__ __forceinline__ int mask_bytes(int chunk, bool prefilter) {
   const int n_it = n_iterations(chunk >> 2);
-  return n_it > 1 ? n_it * kSelThreads * 4 : 0;
+  return prefilter && n_it > 1 ? n_it * kSelThreads * 4 : 0;
 }
 
 // The eight vectors of iteration `it` of this thread, all loads issued before any use.  Missing ones read as
@@ -778,7 +779,7 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   SelShared &sh = *reinterpret_cast<SelShared *>(smem_raw);
   float *staged = reinterpret_cast<float *>(smem_raw + sizeof(SelShared));
   unsigned char *masks = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
-  unsigned char *after = masks + mask_bytes(chunk);
+  unsigned char *after = masks + mask_bytes(chunk, try_fast != 0);
   SelCtx c;
   c.cs = cs; c.rank = rank; c.row = cid; c.chunk = chunk;
   c.lo = rank * chunk;
@@ -1024,7 +1025,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_finalize_candidates_kern
   c.list = nullptr;
   c.list_cap = 0;
   unsigned char *masks = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
-  c.scratch = masks + mask_bytes(chunk);
+  c.scratch = masks + mask_bytes(chunk, true);
   c.cand_cap = cand_cap;
   c.masks = reinterpret_cast<uint32_t *>(masks);
   sh.hist_fast[tid] = 0;
@@ -1122,14 +1123,14 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_finalize_candidates_kern
   SAGEKV_TRACE_END(sp.scores);
 }
 
-static size_t select_smem_bytes(int chunk, int list_cap, int cand_cap, int share, bool resident) {
+static size_t select_smem_bytes(int chunk, int list_cap, int cand_cap, int share, bool prefilter, bool resident) {
   // fast path: candidates (own, all), one keep flag per candidate, the gather list of the CTA's share of the slots;
   // general path: the histograms, then the gather list (as long as the slice, or k_q)
   size_t scratch = (size_t)cand_cap * (8 + 8) + 16 + (((size_t)cand_cap + 15) & ~(size_t)15) + (size_t)share * sizeof(int2);
   const size_t general = (size_t)kGeneralScratch + (size_t)list_cap * sizeof(int2);
   if (scratch < general) scratch = general;
   scratch = (scratch + 15) & ~(size_t)15;
-  return sizeof(SelShared) + scratch + (size_t)mask_bytes(chunk) + (resident ? (size_t)chunk * sizeof(float) : 0);
+  return sizeof(SelShared) + scratch + (size_t)mask_bytes(chunk, prefilter) + (resident ? (size_t)chunk * sizeof(float) : 0);
 }
 
 cudaError_t select_compact_setup() {
@@ -1151,8 +1152,8 @@ cudaError_t launch_score_finalize_candidates(const ScoreParams &sp, cudaStream_t
   chunk = (chunk + 3) & ~3;
   const int cand_cap = list_cand_cap(sp.list_k_q);
   // two CTAs per SM keep every row's cluster resident at once: stage the slice only while two such CTAs fit
-  const bool resident = select_smem_bytes(chunk, 1, cand_cap, 0, true) <= (size_t)kSelSmemLimit / 2;
-  const size_t smem = select_smem_bytes(chunk, 1, cand_cap, 0, resident);
+  const bool resident = select_smem_bytes(chunk, 1, cand_cap, 0, true, true) <= (size_t)kSelSmemLimit / 2;
+  const size_t smem = select_smem_bytes(chunk, 1, cand_cap, 0, true, resident);
   SelectParams p = {};
   p.E = sp.E;
   p.k_q = sp.list_k_q;
@@ -1202,8 +1203,8 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
                        (2 * (int64_t)p.k_q <= (int64_t)cs * kSelThreads || (sketch && 2 * p.k_q <= kSketchFloats));
   const int cand_cap = try_fast ? (p.k_q + p.k_q / 2 + 256) & ~1 : 0;
   const int share = (p.k_q + cs - 1) / cs;              // slots a CTA writes and gathers on the fast path
-  const bool resident = !sketch && select_smem_bytes(chunk, list_cap, cand_cap, share, true) <= (size_t)kSelSmemLimit;
-  const size_t smem = select_smem_bytes(chunk, list_cap, cand_cap, share, resident);
+  const bool resident = !sketch && select_smem_bytes(chunk, list_cap, cand_cap, share, try_fast != 0, true) <= (size_t)kSelSmemLimit;
+  const size_t smem = select_smem_bytes(chunk, list_cap, cand_cap, share, try_fast != 0, resident);
 
   // The sink, recent and last rows: the row clusters copy them along with the kept rows as long as that is at most
   // kStaticPerWarp rows per warp.  More of them (the window is then a large share of the budget) would queue up behind the
