@@ -1205,6 +1205,8 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   const int share = (p.k_q + cs - 1) / cs;              // slots a CTA writes and gathers on the fast path
   const bool resident = !sketch && select_smem_bytes(chunk, list_cap, cand_cap, share, try_fast != 0, true) <= (size_t)kSelSmemLimit;
   const size_t smem = select_smem_bytes(chunk, list_cap, cand_cap, share, try_fast != 0, resident);
+  // the gather list of a large k_q on long slices may not fit: refused here, before the static rows' kernel has written any
+  if (select && smem > (size_t)kSelSmemLimit) return cudaErrorInvalidValue;
 
   // The sink, recent and last rows: the row clusters copy them along with the kept rows as long as that is at most
   // kStaticPerWarp rows per warp.  More of them (the window is then a large share of the budget) would queue up behind the

@@ -1,5 +1,6 @@
 """Selections at the ends of their range: slices of many iterations that the prefilter does not take (their shared memory may
-not grow with the slice) in every way such a launch comes about.  Bit-exact against the oracle."""
+not grow with the slice) in every way such a launch comes about, and a selection too large for the shared memory, which is
+refused before anything is written.  Bit-exact against the oracle."""
 
 import numpy as np
 import pytest
@@ -52,3 +53,19 @@ def test_more_rows_than_sms_with_the_histogram_hint(B):
 
 def test_a_single_cta_per_candidate_list(B):
     run(B, 1, 1, 1, 1600003, 64, 3, 5, hint=2, overlap=2, layers=2)
+
+
+def test_too_large_a_selection_is_refused_before_anything_is_written(B):
+    E, k_q, S, R = 200000, 26000, 4, 300                         # a window that is copied by a kernel of its own
+    N = S + E + R + 1
+    sk = B.SageKV(1, 1, 128, 1, max_ctx=N, max_len=S + k_q + R + 1)
+    K = torch.ones(1, 1, N, 128, dtype=torch.bfloat16, device="cuda")
+    scores, cache = torch.rand(1, E, device="cuda"), sk.new_layer(S, R, k_q)
+    cache.step.fill_(9)
+    with pytest.raises(B.SagekvError) as e:
+        sk.select_compact(scores, K, K, S, R, k_q, cache)
+    assert e.value.code == B.ERR_CUDA
+    torch.cuda.synchronize()
+    assert sk.status() == 0 and int(cache.step.item()) == 9 and cache.state.len == 0
+    assert not cache.Kc.any() and not cache.Vc.any() and not cache.idx.any()
+    sk.close()
