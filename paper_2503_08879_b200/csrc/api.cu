@@ -19,7 +19,7 @@ struct sagekv_ctx {
   int max_chunks;
   float *decode_partials;   // [B*H_kv, max_splits (clusters per head), kPartialStride]
   int max_splits;
-  int32_t *tickets;         // [B*H_kv + 1], zero between launches; the status word follows them
+  int32_t *tickets;         // [B*H_kv + 1], zero between launches; the status word and the selection's ready word follow them
   int32_t *status;          // one int32: kStatus* bits raised by the kernels
   int last_cuda_error;
   int overlap;              // 0, 1 or 2: see sagekv_set_overlap
@@ -113,8 +113,8 @@ int sagekv_create(sagekv_ctx **out, const sagekv_shape *shape, int64_t max_ctx, 
   cudaError_t e = cudaMalloc(&ctx->score_partials, n_rows * ctx->max_chunks * sizeof(float2));
   if (e == cudaSuccess)
     e = cudaMalloc(&ctx->decode_partials, n_heads * ctx->max_splits * kPartialStride * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->tickets, (n_heads + 2) * sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaMemset(ctx->tickets, 0, (n_heads + 2) * sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->tickets, (n_heads + 3) * sizeof(int32_t));
+  if (e == cudaSuccess) e = cudaMemset(ctx->tickets, 0, (n_heads + 3) * sizeof(int32_t));
   if (e == cudaSuccess) ctx->status = ctx->tickets + n_heads + 1;
   if (e != cudaSuccess) {
     cudaFree(ctx->score_partials);
@@ -232,6 +232,7 @@ int sagekv_select_compact(sagekv_ctx *ctx, const float *scores, int64_t scores_r
   p.H_kv = ctx->shape.n_kv_heads;
   p.B = ctx->shape.batch;
   p.status = ctx->status;
+  p.ready = ctx->status + 1;
   p.sketch = !pooled && ctx->hint == 1;
   p.list = !pooled && ctx->hint == 2 && k == ctx->hint_k;
   p.pdl = ctx->select_overlap;

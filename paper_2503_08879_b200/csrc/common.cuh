@@ -92,6 +92,7 @@ struct SelectParams {
   int32_t *d_step;
   int E, S, R, N, k_q, G, H_q, H_kv, B;
   int32_t *status = nullptr;   // status word of the context, or null
+  int32_t *ready = nullptr;    // word by which the static rows' kernel hands the inputs on; 0 between calls
   bool sketch = false;         // the caller asked for the histograms behind the rows to be used (sagekv_set_select_hint)
   bool list = false;           // the caller vouches for the candidate lists behind the rows (hint mode 2)
   int pdl = 0;                 // 0 waits for its predecessor; 1 also releases its successor early; 2 also select before the dependency wait
@@ -219,6 +220,15 @@ __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepco
 __device__ __forceinline__ uint4 ld_stream_v4(const void *ptr) {
   uint4 v;
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(ptr));
+  return v;
+}
+
+// the same through the coherent path: for a kernel that may read ahead of its own dependency wait
+__device__ __forceinline__ uint4 ld_row_v4(const void *ptr) {
+  uint4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                : "l"(ptr));
   return v;

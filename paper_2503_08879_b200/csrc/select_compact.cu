@@ -122,10 +122,21 @@ constexpr int kStaticThreads = 256;
 constexpr int kStaticStages = 2;          // of four rows
 constexpr int kStaticSmem = (kStaticThreads / 32) * kStaticStages * 4 * 512;
 
+// The selection reads its inputs while this kernel runs, so it cannot take them from a dependency wait of its own: the wait
+// here, which makes the predecessor's writes visible to this grid, a release of p.ready by the thread that waited, and an
+// acquire of it in every CTA of the selection make one chain of causality (a bare early release of the dependent launch
+// promises completion, but no visibility).  The word is 1 only while block 0 runs: a CTA of the selection that finds 0,
+// because it starts later or because another launch has come between the two, waits for the dependency instead.
 __global__ void __launch_bounds__(kStaticThreads, 8) copy_static_kernel(const SelectParams p, int alone) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  wait_for_predecessor();                                // the selection that follows must find its inputs complete as soon as it starts
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  wait_for_predecessor();
+  if (!alone) {
+    if (blockIdx.x == 0) {
+      if (threadIdx.x == 0) asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p.ready), "r"(1) : "memory");
+      __syncthreads();                                   // (the word is set before block 0 agrees to the early release)
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per_head = p.S + p.R + 1, groups = (per_head + 3) >> 2, items = p.B * p.H_kv * groups;
   const int n_warps = (int)gridDim.x * (kStaticThreads / 32);
@@ -163,7 +174,10 @@ __global__ void __launch_bounds__(kStaticThreads, 8) copy_static_kernel(const Se
     issue(it + kStaticStages * n_warps, stage);
     if (++stage == kStaticStages) stage = 0;
   }
-  if (alone && blockIdx.x == 0 && threadIdx.x == 0) *p.d_step = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (alone) *p.d_step = 0;
+    else asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p.ready), "r"(0) : "memory");
+  }
 }
 
 // Geometry shared by the two paths
@@ -190,7 +204,7 @@ __host__ __device__ __forceinline__ int mask_bytes(int chunk, bool prefilter) {
 
 // The eight vectors of iteration `it` of this thread, all loads issued before any use.  Missing ones read as
 // -inf, which is below every threshold and never a maximum.
-// kCoherent: the slice was written earlier in this kernel (by this thread), so the read-only path must not be used.
+// kCoherent: the slice was written earlier in this kernel (by this thread): the loads stay behind those stores.
 template <bool kStaged, bool kCoherent = false>
 __device__ __forceinline__ void load8(const float *data, int n_vec, int it, float4 (&x)[8]) {
   const float ninf = -INFINITY;
@@ -206,7 +220,7 @@ __device__ __forceinline__ void load8(const float *data, int n_vec, int it, floa
         asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
                      : "=f"(x[u].x), "=f"(x[u].y), "=f"(x[u].z), "=f"(x[u].w) : "l"(data + 4 * v) : "memory");
       } else {
-        asm volatile("ld.global.nc.v4.f32 {%0,%1,%2,%3}, [%4];"
+        asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];"
                      : "=f"(x[u].x), "=f"(x[u].y), "=f"(x[u].z), "=f"(x[u].w) : "l"(data + 4 * v));
       }
     }
@@ -776,6 +790,8 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   SAGEKV_TRACE_BEGIN
   SAGEKV_STAMP(0);
   cluster.barrier_arrive();   // completed below: every CTA of the cluster runs before anyone writes into a peer
+  int32_t ready = 0;          // (asked for ahead of the set-up, which hides its trip to L2)
+  if (behind_static && threadIdx.x == 0) asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(ready) : "l"(p.ready) : "memory");
   SelShared &sh = *reinterpret_cast<SelShared *>(smem_raw);
   float *staged = reinterpret_cast<float *>(smem_raw + sizeof(SelShared));
   unsigned char *masks = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
@@ -808,9 +824,9 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   // complete (a request to bring the candidate list into L2 changes nothing a program can observe).  Mode 2 (the
   // caller vouches that the predecessor writes none of this call's inputs) puts the wait off until the first
   // write: selection and the first round of row loads run ahead of it, on the candidate-list path.
-  // behind_static: the predecessor is this call's copy_static_kernel, which has found the inputs complete: nothing
-  // here depends on it, but this kernel's end stands for the whole call's, so it waits before it ends.
-  bool waited = behind_static != 0;
+  // behind_static: the predecessor is this call's copy_static_kernel, on which nothing here depends.  If it says so the
+  // inputs are visible (see there) and the wait is put off to the end: this kernel's end stands for the whole call's.
+  bool waited = behind_static && __syncthreads_or(ready) != 0;
   if (p.pdl) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (!waited && (p.pdl < 2 || list_off < 0)) {
     if (p.pdl && list_off >= 0) {
@@ -828,11 +844,11 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   uint32_t tag0 = 0u, tag1 = 0u;
   if (sketch_off >= 0) {
     const uint32_t *sk = reinterpret_cast<const uint32_t *>(p.scores + (int64_t)c.row * p.row_stride + sketch_off);
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(hint.cnt) : "l"(sk + kSketchBins - 1 - tid));
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(tag0) : "l"(sk + kSketchBins));
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(tag1) : "l"(sk + kSketchBins + 1));
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(hint.bin0) : "l"(sk + kSketchBins + 2));
-    asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(hint.kmax) : "l"(sk + kSketchBins + 3));
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(hint.cnt) : "l"(sk + kSketchBins - 1 - tid));
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(tag0) : "l"(sk + kSketchBins));
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(tag1) : "l"(sk + kSketchBins + 1));
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(hint.bin0) : "l"(sk + kSketchBins + 2));
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(hint.kmax) : "l"(sk + kSketchBins + 3));
   }
   // the candidate list of the score step, if the caller vouches for it: its tag words and this thread's share of
   // the entries (as many as the list can have; which of them count is known once the tag is here)
@@ -842,11 +858,11 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   if (list_off >= 0) {
     const uint32_t *tg = reinterpret_cast<const uint32_t *>(p.scores + (int64_t)c.row * p.row_stride + list_off);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(lt[i]) : "l"(tg + i));
+    for (int i = 0; i < 6; ++i) asm volatile("ld.global.u32 %0, [%1];" : "=r"(lt[i]) : "l"(tg + i));
     const unsigned long long *le_src = reinterpret_cast<const unsigned long long *>(tg + kListTagWords);
 #pragma unroll
     for (int i = 0; i < kListRegs; ++i)
-      if (tid + i * kSelThreads < cand_cap) asm volatile("ld.global.nc.u64 %0, [%1];" : "=l"(le[i]) : "l"(le_src + tid + i * kSelThreads));
+      if (tid + i * kSelThreads < cand_cap) asm volatile("ld.global.u64 %0, [%1];" : "=l"(le[i]) : "l"(le_src + tid + i * kSelThreads));
   }
   if (!resident && sketch_off >= 0 && tid == 0 && c.n_local >= 4) {
     // not staged: ask for the slice to be brought into L2 while the threshold bound is worked out from the hint
@@ -954,14 +970,14 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
     if (has_static) {
       const int64_t src_tok = sr < p.S ? sr : (int64_t)p.E + sr;                 // S + E + (sr - S)
       (void)SAGEKV_OK_INDEX(p.status, src_tok >= 0 && src_tok < p.N);
-      vs = ld_stream_v4(src_base + src_tok * p.ks.token_stride);
+      vs = ld_row_v4(src_base + src_tok * p.ks.token_stride);
     }
 #pragma unroll
     for (int u = 0; u < kRows; ++u) {
       if (u < per_warp && e0 + u < n_list) {
         int pos = c.list[e0 + u].y;
         if (!SAGEKV_OK_INDEX(p.status, pos >= p.S && pos < p.S + p.E)) pos = p.S;
-        v[u] = ld_stream_v4(src_base + (int64_t)pos * p.ks.token_stride);
+        v[u] = ld_row_v4(src_base + (int64_t)pos * p.ks.token_stride);
       }
     }
     if (!waited) {                                         // the first write of this warp
