@@ -785,12 +785,16 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int
   return best > 0.f ? with_traffic(best, heads, L) : 0.f;
 }
 
-// The best launch of decode_stream_kernel: CTAs per head, heads per CTA, and its cost in us (0: none).  Measured over
-// 1 to 600 heads and L = 257 .. 8193: 2 plus 0.025 per CTA of a cluster plus 0.6 per tile of a warp (the ring's three tiles
-// per warp in flight against the latency of a copy); 1.9 more when the launches do not overlap; up to 1.5 more when two
-// launches' CTAs do not fit on the device together (24 heads x 2049 rows over 8 CTAs each 6.7 against 7.7 whole); 0.8 per
-// further head of a CTA; a second wave costs a whole time again.
-static float stream_geometry(int L, int heads, const DeviceInfo &dev, bool overlap, int *split, int *per_cta) {
+// The best launch of decode_stream_kernel: CTAs per head, heads per CTA, and its cost in us (0: none).  Fitted to forced launches
+// of every split, 1 to 128 heads x 125 .. 8193 rows x 1 to 8 query heads per KV head (G).  Overlapping: 1.75 plus 0.017 per CTA of a
+// cluster, 0.47 per tile of a warp (the ring's three tiles per warp in flight against the latency of a copy; 0.6 where a CTA takes
+// whole heads), 0.06 per query head, 0.41 per round of the finishing stage (a thread takes two columns of a head: a cluster of 2 with
+// G = 8 needs two), 0.8 per further head of a CTA; up to 1.1 more when two launches' CTAs do not fit on the device together.  A second
+// wave costs a whole time again.  Not overlapping: 3.9, 0.025, 0.6 and 0.8 in place of these, 1 % per query head beyond four.
+// (Without the terms in G, launches with 7 or 8 query heads were streamed where bringing the cache in whole is faster: us whole /
+// streamed at 16 heads x 1537 rows, G = 8: 4.27 / 4.66, 16 x 765 3.64 / 4.04, 4 x 125 2.94 / 3.26.  Of 1173 launches of that sweep in
+// all overlap modes 48 took over 1.5 % longer than before there were streamed ones, now 24; the mean of all 0.785 of the time, now 0.781.)
+static float stream_geometry(int L, int heads, int G, const DeviceInfo &dev, bool overlap, int *split, int *per_cta) {
   const int n_tiles = (L + 15) / 16;
   if ((int64_t)n_tiles * heads > (int64_t)1 << 30) return 0.f;
   float best = 0.f;
@@ -801,10 +805,11 @@ static float stream_geometry(int L, int heads, const DeviceInfo &dev, bool overl
     const int ctas = s == 1 ? (heads + per - 1) / per : heads * s;
     const int waves = (ctas + cap - 1) / cap;
     const int rounds = (per * ((n_tiles + s - 1) / s) + kStWarps - 1) / kStWarps;
-    float one = 2.f + 0.025f * (float)s + 0.6f * (float)rounds + 0.8f * (float)(per - 1);
-    if (!overlap) one += 1.9f;
+    const int finish = s == 1 ? 0 : (G * (kHeadDim / 2) + s * kStThreads - 1) / (s * kStThreads);   // (s == 1: no such stage)
+    const float one = overlap ? 1.75f + 0.017f * (float)s + (s > 1 ? 0.47f : 0.6f) * (float)rounds + 0.06f * (float)G + 0.41f * (float)finish + 0.8f * (float)(per - 1)
+                              : (3.9f + 0.025f * (float)s + 0.6f * (float)rounds + 0.8f * (float)(per - 1)) * (1.f + 0.01f * (float)(G > 4 ? G - 4 : 0));
     float cost = with_traffic((float)waves * one, heads, L);
-    if (2 * ctas > cap) cost += 0.3f + 1.2f * (float)(2 * (ctas < cap ? ctas : cap) - cap) / (float)cap;
+    if (2 * ctas > cap) cost += (overlap ? 0.13f : 0.3f) + (overlap ? 0.95f : 1.2f) * (float)(2 * (ctas < cap ? ctas : cap) - cap) / (float)cap;
     if (best == 0.f || cost < best) { best = cost; *split = s; *per_cta = per; }
   }
   return best;
@@ -852,7 +857,7 @@ cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStre
   // Caches that fill the SMs more than once, and long ones, are streamed; short ones are brought in whole.  (us per
   // launch whole / streamed, overlapping: 8 heads x 2049 rows 4.1 / 4.7, 8 x 8193 11.0 / 9.4, 64 x 2049 17.4 / 13.4,
   // 256 x 2049 84.8 / 42.8)
-  const float stream_cost = tc ? 0.f : stream_geometry(p.L, p.B * p.H_kv, dev, overlap, &split, &heads_per_cta);
+  const float stream_cost = tc ? 0.f : stream_geometry(p.L, p.B * p.H_kv, p.G, dev, overlap, &split, &heads_per_cta);
   const bool streamed = stream_cost > 0.f && cost > 0.f && stream_cost < cost;
   CUtensorMap map_k, map_v;
   if (!make_cache_map(&map_k, p.Kc, p) || !make_cache_map(&map_v, p.Vc, p)) return cudaErrorInvalidValue;
