@@ -286,6 +286,7 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
     __syncthreads();
     SAGEKV_STAMP(5);
     const int64_t row0 = (int64_t)b * p.H_q + kvh * p.G;   // the head's first row of out and lse
+    const bool rows_ok = SAGEKV_OK_INDEX(p.status, b >= 0 && b < p.B && kvh >= 0 && (kvh + 1) * p.G <= p.H_q);
     for (int item = tid; item < p.G * (kHeadDim / 4); item += kStThreads) {
       const int h = item >> 5, col = (item & 31) * 4;
       float2 ml[kStWarps];
@@ -303,9 +304,10 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
       }
       if (split == 1) {
         const float inv = l > 0.f ? 1.f / l : 0.f;
-        *reinterpret_cast<uint2 *>(p.out + (row0 + h) * kHeadDim + col) =
-            make_uint2(pack_bf16x2(o.x * inv, o.y * inv), pack_bf16x2(o.z * inv, o.w * inv));
-        if (p.lse != nullptr && col == 0) p.lse[row0 + h] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
+        if (rows_ok)
+          *reinterpret_cast<uint2 *>(p.out + (row0 + h) * kHeadDim + col) =
+              make_uint2(pack_bf16x2(o.x * inv, o.y * inv), pack_bf16x2(o.z * inv, o.w * inv));
+        if (rows_ok && p.lse != nullptr && col == 0) p.lse[row0 + h] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
       } else {
         // to the CTA that finishes these columns, data and byte count travelling together
         const uint32_t own = (uint32_t)(col >> cols_log);
@@ -347,8 +349,9 @@ decode_stream_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap m
           ox += v[s].x * f; oy += v[s].y * f;
         }
         const float inv = l > 0.f ? 1.f / l : 0.f;
-        *reinterpret_cast<uint32_t *>(p.out + (row0 + h) * kHeadDim + col) = pack_bf16x2(ox * inv, oy * inv);
-        if (p.lse != nullptr && col == 0) p.lse[row0 + h] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
+        const bool ok = rows_ok && SAGEKV_OK_INDEX(p.status, h < p.G && col >= 0 && col + 2 <= kHeadDim);
+        if (ok) *reinterpret_cast<uint32_t *>(p.out + (row0 + h) * kHeadDim + col) = pack_bf16x2(ox * inv, oy * inv);
+        if (ok && p.lse != nullptr && col == 0) p.lse[row0 + h] = l > 0.f ? (M + log2f(l)) * kLn2 : -INFINITY;
       }
     }
     if (++kvh == p.H_kv) { kvh = 0; ++b; }

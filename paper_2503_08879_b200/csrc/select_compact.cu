@@ -167,9 +167,11 @@ __global__ void __launch_bounds__(kStaticThreads, 8) copy_static_kernel(const Se
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int r = r0 + u, row = r < p.S ? r : p.G * p.k_q + r;             // S + G*k_q + (r - S)
+      const int tok = r < p.S ? r : p.E + r;                                 // (a row that was not fetched is not stored)
       uint4 v;
       asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(ring + (uint32_t)(stage * 2048 + u * 512)));
-      if (r < per_head) st_v4(dst + (int64_t)row * p.cs.token_stride, v);
+      if (r < per_head && SAGEKV_OK_INDEX(p.status, tok >= 0 && tok < p.N && row >= 0 && row < p.S + p.G * p.k_q + p.R + 1))
+        st_v4(dst + (int64_t)row * p.cs.token_stride, v);
     }
     issue(it + kStaticStages * n_warps, stage);
     if (++stage == kStaticStages) stage = 0;
@@ -1249,5 +1251,26 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
 }
 
 }  // namespace sagekv
+
+#if defined(SAGEKV_CHECKS)
+// The static rows' kernel alone, with extents the entry points cannot be brought to hand it: `n_ctx` may be less than the
+// positions it would copy.  One KV head, rows of 128 contiguous elements; what K, V, Kc and Vc point at must hold every
+// position and row all the same.
+extern "C" int sagekv_checked_copy_static(const void *K, const void *V, void *Kc, void *Vc, int n_ctx, int n_init, int n_evicted,
+                                          int n_recent, int n_sel, int32_t *d_step, int32_t *status, void *stream) {
+  sagekv::SelectParams p = {};
+  p.K = static_cast<const uint16_t *>(K);
+  p.V = static_cast<const uint16_t *>(V);
+  p.Kc = static_cast<uint16_t *>(Kc);
+  p.Vc = static_cast<uint16_t *>(Vc);
+  p.ks.token_stride = p.cs.token_stride = sagekv::kHeadDim;
+  p.E = n_evicted; p.S = n_init; p.R = n_recent; p.N = n_ctx; p.k_q = n_sel;
+  p.G = p.H_q = p.H_kv = p.B = 1;
+  p.d_step = d_step;
+  p.status = status;
+  return (int)sagekv::launch_next(sagekv::copy_static_kernel, dim3(2), sagekv::kStaticThreads, sagekv::kStaticSmem,
+                                  static_cast<cudaStream_t>(stream), 0, p, 1);
+}
+#endif
 
 SAGEKV_TRACE_READER(sagekv_trace_read_select)
