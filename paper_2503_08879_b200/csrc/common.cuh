@@ -211,9 +211,12 @@ __device__ __forceinline__ void note_bad_index(int32_t *status) {
 }
 
 // The library's kernels are launched as programmatic dependent launches (launch_next): a kernel may be set up while its
-// predecessor on the stream drains.  They begin with this wait, which returns when the predecessor is complete and
-// its writes are visible, so nothing but the launch latency moves; and unless a mode of the interface says so they do
-// not release their own successor before they end.
+// predecessor on the stream drains.  Outside the overlap modes 2 they begin with this wait, which returns when the
+// predecessor is complete and its writes are visible, so nothing but the launch latency moves.  Most release their own
+// successor by ending.  Early, but after the wait, so that whatever came before them is complete and a successor that reads ahead of
+// its own wait can only meet them: the decode kernels that bring a cache in whole (in every overlap mode), decode_stream_kernel
+// (modes 1 and 2), copy_static_kernel (to the selection of the same call).  Before the wait: select_compact_kernel in modes 1
+// and 2, and only there.
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // 16-byte read-only load that does not linger in L1: cache rows are streamed once.
