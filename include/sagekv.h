@@ -181,7 +181,10 @@ int sagekv_decode_attn(sagekv_ctx *ctx, const void *q, const void *k_new, const 
  *      sagekv_decode_attn call on the stream does not write the Kc / Vc passed
  *      to that call (for example a decode call for another layer, or work that
  *      only produces q, k_new, v_new).  q, k_new, v_new and the step counter
- *      are still read after the wait.
+ *      are still read after the wait.  (A call directly behind a select call of
+ *      the same context that was itself launched ahead, sagekv_set_select_overlap,
+ *      runs as in mode 1.  Behind one of another context that guarantee has to
+ *      cover the kernel before it, too.)
  * Errors: INVALID for a null context or a mode outside 0..2. */
 int sagekv_set_overlap(sagekv_ctx *ctx, int mode);
 

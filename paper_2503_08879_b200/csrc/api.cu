@@ -24,6 +24,7 @@ struct sagekv_ctx {
   int last_cuda_error;
   int overlap;              // 0, 1 or 2: see sagekv_set_overlap
   int select_overlap;       // 0, 1 or 2: see sagekv_set_select_overlap
+  bool select_ahead;        // the last select call releases its successor before it has waited for its own predecessor
   int decode_variant;       // 0, 1 or 2: see sagekv_set_decode_variant
   int hint;                 // 0, 1, 2: see sagekv_set_select_hint
   int32_t hint_k;
@@ -91,6 +92,7 @@ int sagekv_create(sagekv_ctx **out, const sagekv_shape *shape, int64_t max_ctx, 
   ctx->last_cuda_error = 0;
   ctx->overlap = 0;
   ctx->select_overlap = 0;
+  ctx->select_ahead = false;
   ctx->decode_variant = 0;
   ctx->hint = 0;
   ctx->hint_k = 0;
@@ -238,6 +240,7 @@ int sagekv_select_compact(sagekv_ctx *ctx, const float *scores, int64_t scores_r
   p.pdl = ctx->select_overlap;
   const cudaError_t e = launch_select_compact(p, ctx->dev->n_sm, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(ctx, e);
+  ctx->select_ahead = p.pdl > 0 && p.list;
   state->n_init = n_init;
   state->k_q = (int32_t)k_q;
   state->n_sel = (int32_t)(G * k_q);
@@ -286,7 +289,11 @@ int sagekv_decode_attn(sagekv_ctx *ctx, const void *q, const void *k_new, const 
   p.H_kv = ctx->shape.n_kv_heads;
   p.B = ctx->shape.batch;
   p.scale_log2 = ctx->scale * kLog2e;
-  p.pdl_mode = ctx->overlap;
+  // In mode 2 the cache is read once the kernel before this one has started.  Behind such a select call the one before that
+  // may still be writing this very cache (two layers: select 0, select 1, decode 0), so this launch waits first.
+  p.pdl_mode = ctx->overlap == 2 && ctx->select_ahead ? 1 : ctx->overlap;
+  p.overlapping = ctx->overlap == 2;                     // (the kernel is chosen as in the calls around it: the same rounding)
+  ctx->select_ahead = false;
   p.variant = ctx->decode_variant == 0 ? kDecodeDefaultVariant : ctx->decode_variant;
   p.pooled = pooled ? 1 : 0;
   const cudaError_t e = launch_decode(p, *ctx->dev, static_cast<cudaStream_t>(stream));

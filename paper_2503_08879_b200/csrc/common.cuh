@@ -149,6 +149,7 @@ struct DecodeParams {
   int S, k_q, n_sel, ring_len, L, G, H_q, H_kv, B;
   float scale_log2;
   int pdl_mode;            // 0 waits for its predecessor, 1 also releases its successor early, 2 also fetch the cache before the wait
+  bool overlapping;        // the launch geometry is chosen for mode 2
   int variant;             // 1 warp-level mma kernel; 2 tensor-memory kernel where it applies
   int pooled;              // 1: every query head sees all selected rows of its KV head (k_q = n_sel), 0: its own segment
 };

@@ -851,7 +851,7 @@ static bool make_cache_map(CUtensorMap *map, const uint16_t *base, const DecodeP
 
 cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStream_t stream) {
   int n_clusters, cs, per_cta, smem, split = 1, heads_per_cta = 1;
-  const bool overlap = p.pdl_mode == 2;
+  const bool overlap = p.overlapping;
   const float cost = decode_geometry(p.L, p.B * p.H_kv, &dev, overlap, &n_clusters, &cs, &per_cta, &smem);
   const bool tc = p.variant == 2 && n_clusters == 1 && per_cta <= kTcMaxTiles;
   // Caches that fill the SMs more than once, and long ones, are streamed; short ones are brought in whole.  (us per

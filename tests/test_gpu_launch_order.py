@@ -1,6 +1,7 @@
 """What a call finds when the kernel directly before it on the stream has written its inputs, where the selection reads them
 while its own static rows are copied by a kernel beside it; alone, and with calls of another context put on the same stream
-from a second thread, between a call's launches too.  Bit-exact against the same calls one at a time."""
+from a second thread, between a call's launches too.  And a decode that reads its cache ahead, behind two select calls that
+run ahead.  Bit-exact against the same calls one at a time."""
 
 import threading
 
@@ -98,4 +99,41 @@ def test_another_context_on_the_same_stream(B):
     assert not errors and int(bad) == 0 and s.sk.status() == 0 and sk.status() == 0
     assert torch.equal(caches[0].idx, caches[1].idx) and torch.equal(caches[0].Kc, caches[1].Kc)
     s.sk.close()
+    sk.close()
+
+
+@pytest.mark.parametrize("kq2,heads", [(20, 1), (300, 2), (1000, 8)])
+def test_decode_behind_two_select_calls_that_run_ahead(B, kq2, heads):
+    n, s0, r0, layers = 16500, 4, 60, 2
+    gen = torch.Generator(device="cuda").manual_seed(kq2)
+    rnd = lambda *s: torch.randn(*s, generator=gen, device="cuda").to(torch.bfloat16)
+    sk = B.SageKV(4 * heads, heads, 128, 1, max_ctx=n, max_len=s0 + 4 * kq2 + r0 + 1)
+    sk.set_select_hint(2, 4 * kq2)
+    K, V = rnd(layers, 1, heads, n, 128), rnd(layers, 1, heads, n, 128)
+    q, kn, vn = rnd(layers, 1, 4 * heads, 128), rnd(layers, 1, heads, 128), rnd(layers, 1, heads, 128)
+    scores = [sk.score(q[l], K[l], s0, r0) for l in range(layers)]
+    caches, out = [sk.new_layer(s0, r0, 4 * kq2) for _ in range(layers)], torch.empty_like(q)
+
+    def calls(between=lambda: None):
+        for l in range(layers):
+            sk.select_compact(scores[l], K[l], V[l], s0, r0, 4 * kq2, caches[l])
+            between()
+        for l in range(layers):
+            sk.decode_attn(q[l], kn[l], vn[l], caches[l], out[l])
+            between()
+
+    sk.set_select_overlap(2)
+    sk.set_overlap(2)
+    calls(torch.cuda.synchronize)
+    want = out.clone()
+    bad = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(50):
+        for c in caches:
+            c.Kc.fill_(3.0)
+            c.Vc.fill_(float("nan"))
+        out.zero_()
+        calls()
+        bad += (out != want).any()
+    torch.cuda.synchronize()
+    assert int(bad) == 0 and sk.status() == 0
     sk.close()
