@@ -26,7 +26,7 @@ lib = C.CDLL(_LIB_PATH)
 try:
     from . import _marshal
 except ImportError as e:
-    raise ImportError("paper_2503_08879_b200/_marshal.so is missing: build it with "
+    raise ImportError("paper_2503_08879_b200/_marshal is missing for this interpreter: build it with "
                       "`python -m paper_2503_08879_b200.build`") from e
 
 OK, ERR_INVALID, ERR_ALIGN, ERR_UNSUPPORTED, ERR_CUDA, ERR_NOMEM = 0, -1, -2, -3, -4, -5

@@ -13,7 +13,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsagekv.so")
 LIB_CHECKED = os.path.join(HERE, "libsagekv_checked.so")   # the same interface built with -DSAGEKV_CHECKS
-MARSHAL = os.path.join(HERE, "_marshal.so")                # argument marshalling of the Python binding's hot calls
+# argument marshalling of the Python binding's hot calls; it uses the interpreter's own interface, so the name carries its tag
+MARSHAL = os.path.join(HERE, "_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
 LIB_TRACE = os.path.join(HERE, "libsagekv_trace.so")       # built with -DSAGEKV_TRACE: timeline stamps in the decode kernel
 SOURCES = ["api.cu", "score.cu", "score_static.cu", "select_compact.cu", "decode_attn.cu", "variants.cu"]
 
@@ -30,6 +31,9 @@ def build_marshal(force: bool = False) -> str:
     deps = [src, os.path.join(ROOT, "include", "sagekv.h")]
     if not force and os.path.exists(MARSHAL) and all(os.path.getmtime(d) <= os.path.getmtime(MARSHAL) for d in deps):
         return MARSHAL
+    untagged = os.path.join(HERE, "_marshal.so")           # as it was once called: any interpreter would take it for its own
+    if os.path.exists(untagged):
+        os.remove(untagged)
     cxx = os.environ.get("CXX") or shutil.which("g++") or "c++"
     cmd = [cxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", os.path.join(ROOT, "include"),
            "-o", MARSHAL, src]

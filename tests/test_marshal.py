@@ -84,3 +84,10 @@ def test_wrong_arguments_raise(recorded):
     with pytest.raises(TypeError):
         m.score(ctx)
     assert got == []
+
+
+def test_the_module_belongs_to_this_interpreter():
+    """Another Python version must not take the module for its own: its name carries the tag of the one it was built for."""
+    import sysconfig
+    from paper_2503_08879_b200 import binding as B
+    assert B._marshal.__file__.endswith("_marshal" + sysconfig.get_config_var("EXT_SUFFIX"))
