@@ -1,4 +1,4 @@
-"""Block bounds at the edges of the kernel's 16-block tiles and 128-block CTAs, for every group size, on summaries as
+"""Block bounds at the edges of the kernel's 16-block tiles and 64-block CTAs, for every group size, on summaries as
 sagekv_quest_build leaves them and on arrays that are no minima and maxima (the formula holds for those too), with
 infinities and zeros.  Tolerance: 128 fp32 additions of exact products, 128 * 2^-24 < 1e-5 of the sum of their magnitudes."""
 
@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("G", [1, 2, 3, 4, 7, 8])
 @pytest.mark.parametrize("n_blocks,ordered,special", [(1, True, False), (15, True, False), (16, True, False), (17, False, False),
-                                                      (127, True, True), (128, False, True), (300, True, False)])
+                                                      (63, False, False), (64, True, True), (65, True, False), (127, True, True), (128, False, True), (300, True, False)])
 def test_bounds_match_the_formula(G, n_blocks, ordered, special):
     from paper_2503_08879_b200 import binding as B
     Bt, Hkv = 2, 3
