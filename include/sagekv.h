@@ -220,7 +220,9 @@ int sagekv_set_decode_variant(sagekv_ctx *ctx, int variant);
  *      for example the select call of another layer, when the score calls of all
  *      layers were queued first.
  * Launches that do not start from a candidate list (select hint modes 0 and 1)
- * pass over the score rows and are always as in mode 0, whatever the mode.
+ * pass over the score rows and are always as in mode 0, whatever the mode.  So
+ * are calls whose sink and recent rows are many (n_init + n_recent + 1 above 32
+ * G times the CTAs per score row, 1 to 8): a kernel beside the selection copies them.
  * Errors: INVALID for a null context or a mode outside 0..2. */
 int sagekv_set_select_overlap(sagekv_ctx *ctx, int mode);
 

@@ -127,6 +127,8 @@ constexpr int kStaticSmem = (kStaticThreads / 32) * kStaticStages * 4 * 512;
 // acquire of it in every CTA of the selection make one chain of causality (a bare early release of the dependent launch
 // promises completion, but no visibility).  The word is 1 only while block 0 runs: a CTA of the selection that finds 0,
 // because it starts later or because another launch has come between the two, waits for the dependency instead.
+// (The trip for the word, us per launch without / with: 64 score rows of 25236, 6145 static rows per head, 33.8 / 33.9, behind
+// the score step 62.1 / 63.2; 32 rows of 124927 26.9 / 28.2.)
 __global__ void __launch_bounds__(kStaticThreads, 8) copy_static_kernel(const SelectParams p, int alone) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   wait_for_predecessor();
