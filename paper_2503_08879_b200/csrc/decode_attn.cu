@@ -793,7 +793,7 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int
 // wave costs a whole time again.  Not overlapping: 3.9, 0.025, 0.6 and 0.8 in place of these, 1 % per query head beyond four.
 // (Without the terms in G, launches with 7 or 8 query heads were streamed where bringing the cache in whole is faster: us whole /
 // streamed at 16 heads x 1537 rows, G = 8: 4.27 / 4.66, 16 x 765 3.64 / 4.04, 4 x 125 2.94 / 3.26.  Of 1173 launches of that sweep in
-// all overlap modes 48 took over 1.5 % longer than before there were streamed ones, now 24; the mean of all 0.785 of the time, now 0.781.)
+// all overlap modes 49 took over 1.5 % longer than before there were streamed ones, now 27; the mean of all 0.787 of the time, now 0.784.)
 static float stream_geometry(int L, int heads, int G, const DeviceInfo &dev, bool overlap, int *split, int *per_cta) {
   const int n_tiles = (L + 15) / 16;
   if ((int64_t)n_tiles * heads > (int64_t)1 << 30) return 0.f;
