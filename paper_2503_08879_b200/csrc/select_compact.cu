@@ -1,7 +1,8 @@
 // Step 2 (second half) and Step 3: per-query-head top-k over the score rows, then the gather that
 // builds the reduced cache  C = Concat(sink, selected, recent, last).
 //
-// One thread-block cluster (up to 8 CTAs) owns one score row.  Each CTA stages its contiguous slice of
+// Rows that fit the registers of one CTA are selected without any exchange (select_short.cuh).  The others:
+// one thread-block cluster (up to 8 CTAs) owns one score row.  Each CTA stages its contiguous slice of
 // the row in shared memory once (cp.async, 16 bytes per request); every later step works on that copy, so
 // the scores cross the memory system a single time.  When the row carries the group maxima of the score
 // step (see common.cuh) the slice is needed only once: it is not staged but requested into L2 with one bulk
@@ -182,6 +183,13 @@ __global__ void __launch_bounds__(kStaticThreads, 8) copy_static_kernel(const Se
     if (alone) *p.d_step = 0;
     else asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p.ready), "r"(0) : "memory");
   }
+}
+
+static cudaError_t launch_copy_static(const SelectParams &p, int n_sm, cudaStream_t stream, bool alone) {
+  const int items = p.B * p.H_kv * ((p.S + p.R + 1 + 3) / 4), per_cta = kStaticThreads / 32 * kStaticStages;
+  int ctas = (items + per_cta - 1) / per_cta;
+  if (ctas > n_sm) ctas = n_sm;
+  return launch_next(copy_static_kernel, dim3((unsigned)ctas), kStaticThreads, kStaticSmem, stream, 0, p, (int)alone);
 }
 
 // Geometry shared by the two paths
@@ -557,10 +565,9 @@ __device__ int fast_candidates(cg::cluster_group &cluster, SelShared &sh, const 
 // k_q entries, each >= T0; sh.hist_fast zero, sh.n_border zero).  arrived: the CTA has a cluster arrival pending
 // (from fast_candidates) that has to be waited for before another path may run.  defer_idx: nothing is written to
 // global memory here; the CTA's (slot, position) list in shared memory is all that comes out.
-__device__ int fast_decide(cg::cluster_group &cluster, SelShared &sh, const SelectParams &p, const SelCtx &c, uint32_t T0,
-                           uint32_t kmax, int M, bool arrived, bool defer_idx = false, unsigned long long *tr = nullptr) {
+__device__ int fast_decide(cg::cluster_group &cluster, SelShared &sh, const SelectParams &p, const SelCtx &c, unsigned long long *cand_all,
+                           uint32_t T0, uint32_t kmax, int M, bool arrived, bool defer_idx = false, unsigned long long *tr = nullptr) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  unsigned long long *cand_all = reinterpret_cast<unsigned long long *>(c.scratch) + c.cand_cap;
   unsigned char *flag = reinterpret_cast<unsigned char *>(cand_all + c.cand_cap + 2);
 
   // 4. which candidates are kept (every CTA decides for all of them).  A 512-bin histogram of the candidate
@@ -663,7 +670,7 @@ __device__ int fast_select(cg::cluster_group &cluster, SelShared &sh, const Sele
   int M = 0, my_start = 0;
   const int code = fast_candidates<kStaged, kSketch>(cluster, sh, p, c, hint, entered, 0.f, T0, kmax, M, my_start);
   if (code != kFastDone) return code;
-  return fast_decide(cluster, sh, p, c, T0, kmax, M, true);
+  return fast_decide(cluster, sh, p, c, reinterpret_cast<unsigned long long *>(c.scratch) + c.cand_cap, T0, kmax, M, true);
 }
 
 // ---- general path -------------------------------------------------------------------------------
@@ -778,6 +785,63 @@ __device__ void general_select(cg::cluster_group &cluster, SelShared &sh, const 
   cluster.sync();   // no CTA moves on (and may exit) while a peer still reads its shared memory
 }
 
+// ---- the gather ---------------------------------------------------------------------------------
+// Copies the rows on a CTA's list into query head j's segment of KV head kvh's reduced cache: a warp moves kRows rows at a time
+// (K in lanes 0-15, V in lanes 16-31), all loads issued before the stores.  rank of cs: the CTA among those of the score row.
+// waited: the dependency wait is over; where it is not, it comes before the first store.
+template <int kRows>
+__device__ __forceinline__ void gather_rows(const SelectParams &p, int b, int kvh, int j, int cs, int rank, const int2 *list, int n_list_all,
+                                            int behind_static, bool &waited) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool gather = p.Kc != nullptr;                   // null: the caller wants the indices only
+  const int n_list = gather ? n_list_all : 0;
+  const uint16_t *src_base = (lane < 16 ? p.K : p.V) + (int64_t)b * p.ks.batch_stride + (int64_t)kvh * p.ks.head_stride +
+                             (lane & 15) * 8;
+  uint16_t *dst_base = (lane < 16 ? p.Kc : p.Vc) + (int64_t)b * p.cs.batch_stride + (int64_t)kvh * p.cs.head_stride +
+                       ((int64_t)p.S + (int64_t)j * p.k_q) * p.cs.token_stride + (lane & 15) * 8;
+  // The sink, recent and last rows of the KV head (positions known without the scores) are shared out over the
+  // warps of the head's G clusters, at most one row per warp per round, loaded together with the first batch.
+  const int n_static = gather && !behind_static ? p.S + p.R + 1 : 0;
+  const int static_stride = p.G * cs * kSelWarps;
+  int sr = (j * cs + rank) * kSelWarps + warp;           // this warp's first static row
+  const int per_warp = n_list > kSelWarps * 4 ? kRows : 4;   // a short list is spread over all the warps
+  for (int e0 = warp * per_warp; e0 < n_list || sr < n_static; e0 += kSelWarps * per_warp) {
+    uint4 v[kRows], vs = make_uint4(0u, 0u, 0u, 0u);
+    const bool has_static = sr < n_static;
+    if (has_static) {
+      const int64_t src_tok = sr < p.S ? sr : (int64_t)p.E + sr;                 // S + E + (sr - S)
+      (void)SAGEKV_OK_INDEX(p.status, src_tok >= 0 && src_tok < p.N);
+      vs = ld_row_v4(src_base + src_tok * p.ks.token_stride);
+    }
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) {
+      if (u < per_warp && e0 + u < n_list) {
+        int pos = list[e0 + u].y;
+        if (!SAGEKV_OK_INDEX(p.status, pos >= p.S && pos < p.S + p.E)) pos = p.S;
+        v[u] = ld_row_v4(src_base + (int64_t)pos * p.ks.token_stride);
+      }
+    }
+    if (!waited) {                                         // the first write of this warp
+      wait_for_predecessor();
+      waited = true;
+    }
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) {
+      if (u < per_warp && e0 + u < n_list) {
+        int slot = list[e0 + u].x;
+        if (!SAGEKV_OK_INDEX(p.status, slot >= 0 && slot < p.k_q)) slot = 0;
+        st_v4(dst_base + (int64_t)slot * p.cs.token_stride, v[u]);
+      }
+    }
+    if (has_static) {
+      // dst_base points at the head's segment S + j*k_q; static rows are addressed from row 0 of the KV head
+      const int64_t dst_row = sr < p.S ? sr : (int64_t)p.G * p.k_q + sr;         // S + G*k_q + (sr - S)
+      st_v4(dst_base + (dst_row - ((int64_t)p.S + (int64_t)j * p.k_q)) * p.cs.token_stride, vs);
+      sr += static_stride;
+    }
+  }
+}
+
 // kAhead: the instance for launches that start from a trusted candidate list with the dependency wait put off
 // (eight rows in flight per warp, which the other instance has no registers for).
 // (The launch bound of the other instance is 64 threads more than it has: that leaves it 56 registers, and the
@@ -810,7 +874,7 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   c.cand_cap = cand_cap;
   c.masks = reinterpret_cast<uint32_t *>(masks);
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int b = c.row / p.H_q, h = c.row - b * p.H_q;
   const int kvh = h / p.G, j = h - kvh * p.G;
   const float *grow = p.scores + (int64_t)c.row * p.row_stride + c.lo;   // 16-byte aligned: chunk % 4 == 0
@@ -917,9 +981,9 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
       __syncthreads();
       SAGEKV_STAMP(2);
 #if defined(SAGEKV_TRACE)
-      code = fast_decide(cluster, sh, p, c, lt[4], lt[5], M, false, !waited, trace_t);
+      code = fast_decide(cluster, sh, p, c, cand_all, lt[4], lt[5], M, false, !waited, trace_t);
 #else
-      code = fast_decide(cluster, sh, p, c, lt[4], lt[5], M, false, !waited);
+      code = fast_decide(cluster, sh, p, c, cand_all, lt[4], lt[5], M, false, !waited);
 #endif
       SAGEKV_STAMP(6);
       idx_deferred = !waited && code == kFastDone;
@@ -951,58 +1015,9 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
     general_select(cluster, sh, p, c);
   }
 
-  // gather the rows on this CTA's list into head j's segment of the reduced cache: a warp moves eight rows at a
-  // time (K in lanes 0-15, V in lanes 16-31), all loads issued before the stores
-  const bool gather = p.Kc != nullptr;                   // null: the caller wants the indices only
-  int32_t *idx_row = p.idx + (int64_t)c.row * p.k_q;
   const int n_list_all = min(sh.list_count, list_cap);
-  const int n_list = gather ? n_list_all : 0;
-  const uint16_t *src_base = (lane < 16 ? p.K : p.V) + (int64_t)b * p.ks.batch_stride + (int64_t)kvh * p.ks.head_stride +
-                             (lane & 15) * 8;
-  uint16_t *dst_base = (lane < 16 ? p.Kc : p.Vc) + (int64_t)b * p.cs.batch_stride + (int64_t)kvh * p.cs.head_stride +
-                       ((int64_t)p.S + (int64_t)j * p.k_q) * p.cs.token_stride + (lane & 15) * 8;
-  // The sink, recent and last rows of the KV head (positions known without the scores) are shared out over the
-  // warps of the head's G clusters, at most one row per warp per round, loaded together with the first batch.
-  const int n_static = gather && !behind_static ? p.S + p.R + 1 : 0;
-  const int static_stride = p.G * cs * kSelWarps;
-  int sr = (j * cs + rank) * kSelWarps + warp;           // this warp's first static row
-  constexpr int kRows = kAhead ? 8 : 4;                    // rows a warp has in flight: all loads issued before the stores
-  const int per_warp = n_list > kSelWarps * 4 ? kRows : 4;   // a short list is spread over all the warps
-  for (int e0 = warp * per_warp; e0 < n_list || sr < n_static; e0 += kSelWarps * per_warp) {
-    uint4 v[kRows], vs = make_uint4(0u, 0u, 0u, 0u);
-    const bool has_static = sr < n_static;
-    if (has_static) {
-      const int64_t src_tok = sr < p.S ? sr : (int64_t)p.E + sr;                 // S + E + (sr - S)
-      (void)SAGEKV_OK_INDEX(p.status, src_tok >= 0 && src_tok < p.N);
-      vs = ld_row_v4(src_base + src_tok * p.ks.token_stride);
-    }
-#pragma unroll
-    for (int u = 0; u < kRows; ++u) {
-      if (u < per_warp && e0 + u < n_list) {
-        int pos = c.list[e0 + u].y;
-        if (!SAGEKV_OK_INDEX(p.status, pos >= p.S && pos < p.S + p.E)) pos = p.S;
-        v[u] = ld_row_v4(src_base + (int64_t)pos * p.ks.token_stride);
-      }
-    }
-    if (!waited) {                                         // the first write of this warp
-      wait_for_predecessor();
-      waited = true;
-    }
-#pragma unroll
-    for (int u = 0; u < kRows; ++u) {
-      if (u < per_warp && e0 + u < n_list) {
-        int slot = c.list[e0 + u].x;
-        if (!SAGEKV_OK_INDEX(p.status, slot >= 0 && slot < p.k_q)) slot = 0;
-        st_v4(dst_base + (int64_t)slot * p.cs.token_stride, v[u]);
-      }
-    }
-    if (has_static) {
-      // dst_base points at the head's segment S + j*k_q; static rows are addressed from row 0 of the KV head
-      const int64_t dst_row = sr < p.S ? sr : (int64_t)p.G * p.k_q + sr;         // S + G*k_q + (sr - S)
-      st_v4(dst_base + (dst_row - ((int64_t)p.S + (int64_t)j * p.k_q)) * p.cs.token_stride, vs);
-      sr += static_stride;
-    }
-  }
+  int32_t *idx_row = p.idx + (int64_t)c.row * p.k_q;
+  gather_rows<kAhead ? 8 : 4>(p, b, kvh, j, cs, rank, c.list, n_list_all, behind_static, waited);   // (a warp's rows in flight)
   if (!waited || behind_static) wait_for_predecessor();   // (not waited: a warp without a round of the loop)
   if (idx_deferred)                                        // every thread is here, and past the wait
     for (int i = tid; i < n_list_all; i += kSelThreads) {
@@ -1143,6 +1158,12 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_finalize_candidates_kern
   SAGEKV_TRACE_END(sp.scores);
 }
 
+}  // namespace sagekv
+
+#include "select_short.cuh"
+
+namespace sagekv {
+
 static size_t select_smem_bytes(int chunk, int list_cap, int cand_cap, int share, bool prefilter, bool resident) {
   // fast path: candidates (own, all), one keep flag per candidate, the gather list of the CTA's share of the slots;
   // general path: the histograms, then the gather list (as long as the slice, or k_q)
@@ -1162,6 +1183,8 @@ cudaError_t select_compact_setup() {
   e = cudaFuncSetAttribute(select_compact_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(select_compact_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
+  if (e != cudaSuccess) return e;
+  e = select_short_setup();
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(score_finalize_candidates_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
 }
@@ -1190,6 +1213,7 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   // many rows smaller clusters pay, because two CTAs per SM times the SM count is all that runs at once.
   const bool list = select && p.list && list_applies(p.E, p.k_q, p.row_stride);
   const bool sketch = list || (select && p.sketch && sketch_fits(p.E, p.row_stride));   // both read the row unstaged, if at all
+  if (select && !list && short_rows_apply(p, n_sm, sketch)) return launch_select_short(p, n_sm, stream);
   // Cluster size, at most 8 CTAs (the portable limit).
   int cs = 1;
   const int n_static = p.Kc != nullptr ? p.S + p.R + 1 : 0;   // sink, recent and last rows per KV head
@@ -1240,10 +1264,7 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   SelectParams pl = p;
   if (!list || beside) pl.pdl = 0;
   if (beside) {
-    const int items = p.B * p.H_kv * ((n_static + 3) / 4), per_cta = kStaticThreads / 32 * kStaticStages;
-    int ctas = (items + per_cta - 1) / per_cta;
-    if (ctas > n_sm) ctas = n_sm;
-    const cudaError_t e = launch_next(copy_static_kernel, dim3((unsigned)ctas), kStaticThreads, kStaticSmem, stream, 0, pl, (int)!select);
+    const cudaError_t e = launch_copy_static(pl, n_sm, stream, !select);
     if (e != cudaSuccess || !select) return e;
   }
   const int64_t sketch_off = try_fast && sketch && !list ? sketch_offset(p.E) : (int64_t)-1;
