@@ -24,7 +24,8 @@
 //      ascending positions.  Each CTA writes and gathers an even share of the slots.
 // General path (k_q large, tiny rows, or more candidates than the buffers hold, e.g. a row of equal
 // scores): three-digit radix select (11 + 11 + 10 bits) with histograms merged in CTA 0's shared memory by
-// distributed-shared-memory atomics, then a ballot/popcount ranking in row order.
+// distributed-shared-memory atomics, then a ballot/popcount ranking in row order; launches known to need it from the start have
+// a kernel of their own (select_general_kernel).
 // The rows on a CTA's list are then copied into the head's segment of the reduced cache (general path: the
 // CTA that owns a kept element copies it), together with a share of the KV head's sink, recent and last rows.
 #include <cooperative_groups.h>
@@ -60,6 +61,9 @@ struct SelShared {
   int pad_[3];
 };
 static_assert(sizeof(SelShared) % 16 == 0, "staged scores must stay 16-byte aligned");
+
+// the key of a score where one that is no number (NaN) is the smallest, as in the prefilter and in the oracle
+__device__ __forceinline__ uint32_t number_key(float x) { return score_key(fmaxf(x, -INFINITY)); }
 
 __device__ __forceinline__ float key_to_score(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
@@ -673,7 +677,7 @@ __device__ int fast_select(cg::cluster_group &cluster, SelShared &sh, const Sele
   return fast_decide(cluster, sh, p, c, reinterpret_cast<unsigned long long *>(c.scratch) + c.cand_cap, T0, kmax, M, true);
 }
 
-// ---- general path -------------------------------------------------------------------------------
+// ---- general path: as the prefilter's last resort, in the few registers beside it ------------------------
 __device__ void general_select(cg::cluster_group &cluster, SelShared &sh, const SelectParams &p, const SelCtx &c) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t(*hist_merged)[kMaxBins] = reinterpret_cast<uint32_t(*)[kMaxBins]>(c.scratch);   // only rank 0's copy is used
@@ -849,7 +853,7 @@ __device__ __forceinline__ void gather_rows(const SelectParams &p, int b, int kv
 template <bool kAhead>
 __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) select_compact_kernel(const SelectParams p, int behind_static, int chunk,
                                                                       int resident, int list_cap, int cand_cap,
-                                                                      int try_fast, int64_t sketch_off, int64_t list_off) {
+                                                                      int64_t sketch_off, int64_t list_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = cluster.num_blocks();
@@ -863,7 +867,7 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   SelShared &sh = *reinterpret_cast<SelShared *>(smem_raw);
   float *staged = reinterpret_cast<float *>(smem_raw + sizeof(SelShared));
   unsigned char *masks = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
-  unsigned char *after = masks + mask_bytes(chunk, try_fast != 0);
+  unsigned char *after = masks + mask_bytes(chunk, true);
   SelCtx c;
   c.cs = cs; c.rank = rank; c.row = cid; c.chunk = chunk;
   c.lo = rank * chunk;
@@ -965,49 +969,45 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   // The gather list follows the buffers of the path that runs (see select_smem_bytes).
   bool done = false, exit_wait = false;   // exit_wait: a cluster arrival of the prefilter is still to be waited for
   bool idx_deferred = false;              // the selection wrote no indices: they follow from the gather lists
-  if (try_fast) {
-    c.list = reinterpret_cast<int2 *>(c.scratch + (size_t)cand_cap * 16 + 16 + (((size_t)cand_cap + 15) & ~(size_t)15));
-    int code = kFastRetry;
-    if (list_off >= 0 && lt[0] == kListMagic && lt[1] == (uint32_t)p.E && lt[2] == (uint32_t)p.k_q && (int)lt[3] >= p.k_q &&
-        (int)lt[3] <= cand_cap && cand_cap <= kListRegs * kSelThreads) {   // the same words in every CTA of the row
-      // start from the score step's list: no pass over the row, no exchange between the CTAs
-      const int M = (int)lt[3];
-      unsigned long long *cand_all = reinterpret_cast<unsigned long long *>(c.scratch) + cand_cap;
+  c.list = reinterpret_cast<int2 *>(c.scratch + (size_t)cand_cap * 16 + 16 + (((size_t)cand_cap + 15) & ~(size_t)15));
+  int code = kFastRetry;
+  if (list_off >= 0 && lt[0] == kListMagic && lt[1] == (uint32_t)p.E && lt[2] == (uint32_t)p.k_q && (int)lt[3] >= p.k_q &&
+      (int)lt[3] <= cand_cap && cand_cap <= kListRegs * kSelThreads) {   // the same words in every CTA of the row
+    // start from the score step's list: no pass over the row, no exchange between the CTAs
+    const int M = (int)lt[3];
+    unsigned long long *cand_all = reinterpret_cast<unsigned long long *>(c.scratch) + cand_cap;
 #pragma unroll
-      for (int i = 0; i < kListRegs; ++i)
-        if (tid + i * kSelThreads < M) cand_all[tid + i * kSelThreads] = le[i];
-      if (tid == 0) sh.n_border = 0;
-      cluster.barrier_wait();                              // the arrive at kernel entry; no peer's memory is touched on this path
-      __syncthreads();
-      SAGEKV_STAMP(2);
+    for (int i = 0; i < kListRegs; ++i)
+      if (tid + i * kSelThreads < M) cand_all[tid + i * kSelThreads] = le[i];
+    if (tid == 0) sh.n_border = 0;
+    cluster.barrier_wait();                              // the arrive at kernel entry; no peer's memory is touched on this path
+    __syncthreads();
+    SAGEKV_STAMP(2);
 #if defined(SAGEKV_TRACE)
-      code = fast_decide(cluster, sh, p, c, cand_all, lt[4], lt[5], M, false, !waited, trace_t);
+    code = fast_decide(cluster, sh, p, c, cand_all, lt[4], lt[5], M, false, !waited, trace_t);
 #else
-      code = fast_decide(cluster, sh, p, c, cand_all, lt[4], lt[5], M, false, !waited);
+    code = fast_decide(cluster, sh, p, c, cand_all, lt[4], lt[5], M, false, !waited);
 #endif
-      SAGEKV_STAMP(6);
-      idx_deferred = !waited && code == kFastDone;
-      if (code == kFastGeneral) {                          // (a large group of equal scores at the cut)
-        if (!waited) { wait_for_predecessor(); waited = true; }
-        c.list = reinterpret_cast<int2 *>(c.scratch + kGeneralScratch);
-        general_select(cluster, sh, p, c);
-        code = kFastDone;
-      }
-      done = true;
+    SAGEKV_STAMP(6);
+    idx_deferred = !waited && code == kFastDone;
+    if (code == kFastGeneral) {                          // (a large group of equal scores at the cut)
+      if (!waited) { wait_for_predecessor(); waited = true; }
+      c.list = reinterpret_cast<int2 *>(c.scratch + kGeneralScratch);
+      general_select(cluster, sh, p, c);
+      code = kFastDone;
     }
-    if (!done && !waited) { wait_for_predecessor(); waited = true; }   // the other paths write as they go
-    if (!done && sketch_off >= 0 && tag0 == kSketchMagic && tag1 == (uint32_t)p.E)   // the same words in every CTA of the row
-      code = resident ? fast_select<true, true>(cluster, sh, p, c, hint, false)
-                      : fast_select<false, true>(cluster, sh, p, c, hint, false);
-    if (!done) {
-      if (code == kFastRetry || code == kFastRetryEntered)
-        code = resident ? fast_select<true, false>(cluster, sh, p, c, hint, code == kFastRetryEntered)
-                        : fast_select<false, false>(cluster, sh, p, c, hint, code == kFastRetryEntered);
-      done = code == kFastDone;
-      exit_wait = done;
-    }
-  } else {
-    cluster.barrier_wait();
+    done = true;
+  }
+  if (!done && !waited) { wait_for_predecessor(); waited = true; }   // the other paths write as they go
+  if (!done && sketch_off >= 0 && tag0 == kSketchMagic && tag1 == (uint32_t)p.E)   // the same words in every CTA of the row
+    code = resident ? fast_select<true, true>(cluster, sh, p, c, hint, false)
+                    : fast_select<false, true>(cluster, sh, p, c, hint, false);
+  if (!done) {
+    if (code == kFastRetry || code == kFastRetryEntered)
+      code = resident ? fast_select<true, false>(cluster, sh, p, c, hint, code == kFastRetryEntered)
+                      : fast_select<false, false>(cluster, sh, p, c, hint, code == kFastRetryEntered);
+    done = code == kFastDone;
+    exit_wait = done;
   }
   if (!done) {
     if (!waited) { wait_for_predecessor(); waited = true; }
@@ -1030,6 +1030,206 @@ __global__ void __launch_bounds__(kAhead ? kSelThreads : kSelThreads + 64, 2) se
   SAGEKV_STAMP(9);
   SAGEKV_TRACE_END(p.idx);
   if (exit_wait) cluster.barrier_wait();   // prefilter path: a peer may still have been copying this CTA's candidates
+}
+
+// ---- general path: the launches that the prefilter does not take ------------------------------------------
+// Any k_q, any scores: the cut is found by histograms of 2048 bins over ever fewer bits of the keys (of all scores between the
+// row's extremes first), each CTA counting its slice and every CTA adding up all of them over distributed shared memory; then the
+// kept scores are ranked in row order.  Bound by the passes over the slice: their loads are in flight four or eight at a time,
+// where the path above takes one after another, and the bins lie where the scores are.  (us per launch as that path / so: 8 rows x
+// 316197 with k_q = 2399 69.4 / 58.7, 8 x 486254 with 7504 178 / 97, 64 x 51468 with 2758 125 / 86; softmax rows of two heads,
+// 524151 with 8056, 188 / 105.)
+__device__ __forceinline__ void general_select_wide(cg::cluster_group &cluster, SelShared &sh, const SelectParams &p, const SelCtx &c) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t(*hist)[kMaxBins] = reinterpret_cast<uint32_t(*)[kMaxBins]>(c.scratch);   // two, used in turn: peers may still read the last one
+  const float *data = c.data;
+  const int n_local = c.n_local, n_vec = n_local >> 2, tail_i = (n_vec << 2) + tid;
+  asm volatile("cp.async.wait_all;" ::: "memory");       // the staged slice: every thread reads all of it here
+  __syncthreads();
+  auto each_key = [&](auto &&f) {                        // f(key) for all scores of the slice; 0: none (whole warps call it together)
+    for (int v0 = tid; v0 - lane < n_vec; v0 += 4 * kSelThreads) {
+      float4 x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v0 + u * kSelThreads < n_vec) x[u] = *reinterpret_cast<const float4 *>(data + 4 * (v0 + u * kSelThreads));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool is = v0 + u * kSelThreads < n_vec;
+        f(is ? number_key(x[u].x) : 0u); f(is ? number_key(x[u].y) : 0u);
+        f(is ? number_key(x[u].z) : 0u); f(is ? number_key(x[u].w) : 0u);
+      }
+    }
+    if (warp == 0) f(tail_i < n_local ? number_key(data[tail_i]) : 0u);   // the slice's last (n_local % 4) scores
+  };
+
+  // the extremes of the row
+  uint32_t kmin = 0xffffffffu, kmax = 0u;
+  each_key([&](uint32_t k) { kmin = min(kmin, k - 1u); kmax = max(kmax, k); });   // (none: wraps to the largest)
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if (lane == 0) { sh.red[0][warp] = kmin; sh.red[1][warp] = kmax; }
+  if (tid == 0) sh.list_count = 0;
+  *reinterpret_cast<uint4 *>(&hist[0][4 * tid]) = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  if (warp == 0) {
+    kmin = __reduce_min_sync(0xffffffffu, lane < kSelWarps ? sh.red[0][lane] : 0xffffffffu);
+    kmax = __reduce_max_sync(0xffffffffu, lane < kSelWarps ? sh.red[1][lane] : 0u);
+    if (lane < c.cs) {
+      uint32_t *gs = cluster.map_shared_rank(&sh.gstat[0][0], lane) + 4 * c.rank;
+      gs[0] = kmin; gs[1] = kmax;
+    }
+  }
+  cluster.sync();
+  kmin = 0xffffffffu; kmax = 0u;
+  for (int r = 0; r < c.cs; ++r) { kmin = min(kmin, sh.gstat[r][0]); kmax = max(kmax, sh.gstat[r][1]); }
+  ++kmin;
+
+  const uint32_t diff = kmax ^ kmin;
+  int shift = max(0, (diff ? 31 - __clz(diff) : 0) - 10);   // (kmax >> shift) - (kmin >> shift) < 2048
+  uint32_t base = kmin >> shift, cut = 0u;
+  int cut_shift = 0;
+  int wanted = p.k_q;                                    // the score looked for is the `wanted`-th largest of those that are counted
+  for (int level = 0;; ++level) {
+    uint32_t *mine = hist[level & 1];
+    each_key([&](uint32_t k) {
+      const bool in = k >= kmin && (level == 0 || (k >> cut_shift) == cut);
+      const uint32_t bin = in ? (k >> shift) - base : 0xffffffffu;
+      const uint32_t first = __shfl_sync(0xffffffffu, bin, 0);
+      if (__all_sync(0xffffffffu, bin == first)) {       // (a row of equal scores would queue up at one word)
+        if (lane == 0 && in) atomicAdd(&mine[bin], 32u);
+      } else if (in) {
+        atomicAdd(&mine[bin], 1u);
+      }
+    });
+    cluster.sync();
+    int cnt[4] = {0, 0, 0, 0};                           // of the row: thread 0 has the top four bins
+    for (int r = 0; r < c.cs; ++r) {
+      const uint4 c4 = *reinterpret_cast<const uint4 *>(cluster.map_shared_rank(&mine[kMaxBins - 4 - 4 * tid], r));
+      cnt[0] += (int)c4.w; cnt[1] += (int)c4.z; cnt[2] += (int)c4.y; cnt[3] += (int)c4.x;
+    }
+    int before = block_exclusive_scan(cnt[0] + cnt[1] + cnt[2] + cnt[3], sh.scan_tmp);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (before < wanted && before + cnt[e] >= wanted) {
+        sh.found[0] = kMaxBins - 1 - (4 * tid + e); sh.found[1] = wanted - before; sh.wsum[0] = cnt[e];
+      }
+      before += cnt[e];
+    }
+    *reinterpret_cast<uint4 *>(&hist[(level + 1) & 1][4 * tid]) = make_uint4(0u, 0u, 0u, 0u);   // (every peer has read it)
+    __syncthreads();
+    cut = base + (uint32_t)sh.found[0];
+    wanted = sh.found[1];
+    const int in_cut = sh.wsum[0];
+    __syncthreads();                                     // (found[] is rewritten by the next level)
+    cut_shift = shift;
+    if (in_cut == wanted || shift == 0) break;           // (all of the bin's are kept, or they are equal)
+    shift = max(0, shift - 11);
+    base = cut << (cut_shift - shift);
+  }
+
+  // ranks in row order: warp w owns the contiguous range [w*wlen, (w+1)*wlen) of the slice; `wanted` keys of the cut's bin are kept,
+  // lowest positions first (all there are, or equal ones)
+  constexpr int kAtOnce = 8;
+  const int wlen = (((c.chunk + kSelWarps - 1) / kSelWarps) + 31) & ~31;
+  const int wlo = warp * wlen, whi = min(n_local, wlo + wlen);
+  auto in_order = [&](auto &&f) {                        // f(index, key above the cut's bin, key in it) for 32 scores at a time
+    for (int first = wlo; first < whi; first += 32 * kAtOnce) {
+      float x[kAtOnce];
+#pragma unroll
+      for (int u = 0; u < kAtOnce; ++u)
+        if (first + 32 * u + lane < whi) x[u] = data[first + 32 * u + lane];
+#pragma unroll
+      for (int u = 0; u < kAtOnce; ++u) {
+        const int i = first + 32 * u + lane;
+        if (first + 32 * u >= whi) break;
+        const uint32_t k = i < whi ? number_key(x[u]) : 0u;
+        f(i, k >= kmin && (k >> shift) > cut, k >= kmin && (k >> shift) == cut);
+      }
+    }
+  };
+  int n_gt = 0, n_eq = 0;
+  in_order([&](int, bool gt, bool eq) {
+    n_gt += __popc(__ballot_sync(0xffffffffu, gt));
+    n_eq += __popc(__ballot_sync(0xffffffffu, eq));
+  });
+  if (lane == 0) { sh.warp_cnt[warp][0] = n_gt; sh.warp_cnt[warp][1] = n_eq; }
+  __syncthreads();
+  int gt_before = 0, eq_before = 0, cta_gt = 0, cta_eq = 0;
+  for (int w = 0; w < kSelWarps; ++w) {
+    const int a = sh.warp_cnt[w][0], e = sh.warp_cnt[w][1];
+    if (w < warp) { gt_before += a; eq_before += e; }
+    cta_gt += a; cta_eq += e;
+  }
+  if (tid == 0) {
+    int *t0 = cluster.map_shared_rank(&sh.totals[0][0], 0);
+    t0[2 * c.rank] = cta_gt;
+    t0[2 * c.rank + 1] = cta_eq;
+  }
+  cluster.sync();
+  {
+    const int *t0 = cluster.map_shared_rank(&sh.totals[0][0], 0);
+    for (int r = 0; r < c.rank; ++r) { gt_before += t0[2 * r]; eq_before += t0[2 * r + 1]; }
+  }
+
+  int32_t *idx_row = p.idx + (int64_t)c.row * p.k_q;
+  in_order([&](int i, bool gt, bool eq) {
+    const uint32_t bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
+    const uint32_t below = (1u << lane) - 1u;
+    const int g_here = gt_before + __popc(bg & below), e_here = eq_before + __popc(be & below);
+    int slot = -1;
+    if (gt) slot = g_here + min(e_here, wanted);
+    else if (eq && e_here < wanted) slot = g_here + e_here;
+    if (slot >= 0) {
+      const int pos = p.S + c.lo + i;
+      if (SAGEKV_OK_INDEX(p.status, slot < p.k_q && pos < p.S + p.E)) idx_row[slot] = pos;
+      const int n = atomicAdd(&sh.list_count, 1);
+      if (n < c.list_cap) c.list[n] = make_int2(slot, pos);
+    }
+    gt_before += __popc(bg);
+    eq_before += __popc(be);
+  });
+  __syncthreads();
+  cluster.sync();   // no CTA moves on (and may exit) while a peer still reads its shared memory
+}
+
+__global__ void __launch_bounds__(kSelThreads, 2) select_general_kernel(const SelectParams p, int behind_static, int chunk, int resident, int list_cap) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.barrier_arrive();   // every CTA of the cluster runs before anyone writes into a peer
+  int32_t ready = 0;
+  if (behind_static && threadIdx.x == 0) asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(ready) : "l"(p.ready) : "memory");
+  SelShared &sh = *reinterpret_cast<SelShared *>(smem_raw);
+  float *staged = reinterpret_cast<float *>(smem_raw + sizeof(SelShared));
+  const int tid = threadIdx.x;
+  SelCtx c;
+  c.cs = cluster.num_blocks(); c.rank = cluster.block_rank(); c.row = blockIdx.x / c.cs; c.chunk = chunk;
+  c.lo = c.rank * chunk;
+  c.n_local = max(0, min(p.E - c.lo, chunk));
+  c.scratch = smem_raw + sizeof(SelShared) + (resident ? (size_t)chunk * sizeof(float) : 0);
+  c.list = reinterpret_cast<int2 *>(c.scratch + kGeneralScratch);
+  c.list_cap = list_cap;
+  c.cand_cap = 0;
+  c.masks = nullptr;
+  const float *grow = p.scores + (int64_t)c.row * p.row_stride + c.lo;   // 16-byte aligned: chunk % 4 == 0
+  c.data = resident ? staged : grow;
+  const int b = c.row / p.H_q, h = c.row - b * p.H_q, kvh = h / p.G, j = h - kvh * p.G;
+  (void)SAGEKV_OK_INDEX(p.status, c.row < p.B * p.H_q && (int64_t)c.lo + c.n_local <= p.row_stride && c.lo + c.n_local <= p.E);
+  bool waited = behind_static && __syncthreads_or(ready) != 0;   // (see select_compact_kernel)
+  if (!waited) {
+    wait_for_predecessor();
+    waited = true;
+  }
+  if (resident) {
+    const int n_vec = c.n_local >> 2, tail_i = (n_vec << 2) + tid;
+    for (int v = tid; v < n_vec; v += kSelThreads)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(staged + 4 * v)), "l"(grow + 4 * v) : "memory");
+    if (tail_i < c.n_local) staged[tail_i] = grow[tail_i];
+  }
+  cluster.barrier_wait();
+  general_select_wide(cluster, sh, p, c);
+  gather_rows<4>(p, b, kvh, j, c.cs, c.rank, c.list, min(sh.list_count, list_cap), behind_static, waited);
+  if (behind_static) wait_for_predecessor();
+  if (blockIdx.x == 0 && tid == 0 && p.d_step != nullptr) *p.d_step = 0;
 }
 
 // ---- second pass of the score step in hint mode 2 -----------------------------------------------------------
@@ -1184,6 +1384,8 @@ cudaError_t select_compact_setup() {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(select_compact_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(select_general_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
+  if (e != cudaSuccess) return e;
   e = select_short_setup();
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(score_finalize_candidates_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
@@ -1269,8 +1471,10 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   }
   const int64_t sketch_off = try_fast && sketch && !list ? sketch_offset(p.E) : (int64_t)-1;
   const int64_t list_off = try_fast && list ? sketch_offset(p.E) : (int64_t)-1;
+  if (!try_fast)
+    return launch_next(select_general_kernel, dim3((unsigned)(n_rows * cs)), kSelThreads, smem, stream, cs, pl, (int)beside, chunk, (int)resident, list_cap);
   return launch_next(ahead ? select_compact_kernel<true> : select_compact_kernel<false>, dim3((unsigned)(n_rows * cs)), kSelThreads, smem,
-                     stream, cs, pl, (int)beside, chunk, (int)resident, list_cap, cand_cap, try_fast, sketch_off, list_off);
+                     stream, cs, pl, (int)beside, chunk, (int)resident, list_cap, cand_cap, sketch_off, list_off);
 }
 
 }  // namespace sagekv

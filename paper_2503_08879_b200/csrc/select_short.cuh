@@ -20,18 +20,15 @@ constexpr int kShortBins = 2048;
 constexpr int kShortBorder = 32;          // scores of the cut's bin that are ranked one against another
 constexpr int kShortMaxE = 16 * 4 * kSelThreads;
 
-// A number that is none (NaN) is the smallest, as in the prefilter of the long rows.
-__device__ __forceinline__ uint32_t short_key(float x) { return score_key(fmaxf(x, -INFINITY)); }
-
 // Element 4u + e of a thread is element e of vector (warp * kVec + u) * 32 + lane of the row, so that (warp, u, lane, e) order is
 // position order; the first n of a thread's elements exist.  Key 0, below the key of every number, stands for none.
 template <int kVec, bool kKeys>
 struct ShortRow {
   uint32_t w[4 * kVec];                   // keys, or (kKeys = false) scores whose keys are worked out where they are needed
   int n;
-  __device__ __forceinline__ void set(int i, float x) { w[i] = kKeys ? (i < n ? short_key(x) : 0u) : __float_as_uint(x); }
+  __device__ __forceinline__ void set(int i, float x) { w[i] = kKeys ? (i < n ? number_key(x) : 0u) : __float_as_uint(x); }
   __device__ __forceinline__ float score(int i) const { return __uint_as_float(w[i]); }
-  __device__ __forceinline__ uint32_t key(int i) const { return kKeys ? w[i] : (i < n ? short_key(__uint_as_float(w[i])) : 0u); }
+  __device__ __forceinline__ uint32_t key(int i) const { return kKeys ? w[i] : (i < n ? number_key(__uint_as_float(w[i])) : 0u); }
 };
 
 template <int kVec>
