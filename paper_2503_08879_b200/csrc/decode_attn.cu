@@ -4,7 +4,7 @@
 // Flash-decoding on thread-block clusters.  The L rows of one KV head are cut into 16-row tiles that are
 // dealt evenly, as contiguous ranges, to the CTAs of one cluster.  A CTA brings its K and V tiles into shared
 // memory with tensor copies (one 16-row x 64-column box per request, 128-byte swizzle, completion counted on
-// an mbarrier), issued by a ninth warp that does nothing else.  The staging area has 50 slots of one tile
+// an mbarrier), issued by a ninth warp that does nothing else, or by all nine (decode_shares_issue).  The staging area has 50 slots of one tile
 // (K or V) each.  All K tiles of the range are resident from the start; so are the V tiles while slots last,
 // and the remaining V tiles take over the K slots as soon as the first product is done.  There is one pass:
 //   S = K Q^T     16 rows x 8 heads per mma, a tile per warp in turn (the scores of all its tiles stay in
@@ -137,7 +137,7 @@ __device__ __forceinline__ void bar_sync(int id, int n_threads) {
 // n_slots: slots of this launch's staging area (min(2 * most tiles of a CTA, kDecodeSlots)).
 // kLong: a CTA may have more tiles than half the slots (part of V arrives late, a warp may have up to six tiles in
 // the first product); false keeps the common case free of that.
-template <bool kLong>
+template <bool kLong, bool kShared>
 __global__ void __launch_bounds__(kDecodeThreads, 1)
 decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                    const int n_slots) {
@@ -190,6 +190,10 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
     // from every CTA of the cluster: 8 bytes per (own column, head pair in use) and 64 bytes of (max, sum) pairs
     mbar_expect_tx(inbox_bar, (uint32_t)(cs * my_cols * n_pairs * 8));
     mbar_expect_tx(ml_bar, (uint32_t)(cs * 64));
+    if (kShared) {
+      mbar_expect_tx(kbar, (uint32_t)n * kSlotBytes);
+      mbar_expect_tx(vbar_e, (uint32_t)n_early * kSlotBytes);
+    }
   }
   __syncthreads();
   cluster.barrier_arrive();                              // waited for just before the first store into a peer: its barrier is set up
@@ -204,24 +208,35 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
-  // ---- the warp that issues the copies: lane i takes requests i, i + 32, ... (two boxes per tile) ----
+  // ---- the copies, two boxes per tile: requests op_lo + who, op_lo + who + step, ... of a range of tiles ----
+  uint64_t stream_policy;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_policy));
+  auto request = [&](const CUtensorMap *map, int t_lo, int t_hi, bool is_v, uint32_t bar, int who, int step) {   // tiles [t_lo, t_hi)
+    for (int op = 2 * t_lo + who; op < 2 * t_hi; op += step) {
+      const int t = op >> 1, hf = op & 1;
+      const uint32_t dst = stage + (uint32_t)((is_v ? v_slot(t) : t) * kSlotBytes + hf * kHalfBytes);
+      tensor_copy_4d(dst, map, hf * 64, (first_tile + t) << 4, kvh, b, bar, stream_policy);
+    }
+  };
+  if (kShared) {                                         // (the byte counts are set above)
+    const int who = lane * (kDecodeWarps + 1) + (producer ? 0 : warp + 1);
+    request(&map_k, 0, n, false, kbar, who, kDecodeThreads);
+    request(&map_v, 0, n_early, true, vbar_e, who, kDecodeThreads);
+  }
+  // ---- the warp that issues the copies: lane i takes requests i, i + 32, ... ----
   if (producer) {
-    uint64_t stream_policy;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(stream_policy));
     auto issue = [&](const CUtensorMap *map, int t_lo, int t_hi, bool is_v, uint32_t bar) {   // tiles [t_lo, t_hi)
       if (lane == 0 && t_hi > t_lo) mbar_expect_tx(bar, (uint32_t)(t_hi - t_lo) * kSlotBytes);
       __syncwarp();
-      for (int op = lane; op < (t_hi - t_lo) * 2; op += 32) {
-        const int t = t_lo + (op >> 1), hf = op & 1;
-        const uint32_t dst = stage + (uint32_t)((is_v ? v_slot(t) : t) * kSlotBytes + hf * kHalfBytes);
-        tensor_copy_4d(dst, map, hf * 64, (first_tile + t) << 4, kvh, b, bar, stream_policy);
-      }
+      request(map, t_lo, t_hi, is_v, bar, lane, 32);
     };
     // (In prefetch mode this warp never waits for the predecessor: it reads nothing of it, and what it requests
     // after barrier A comes after the consumers' wait.  It leaves the release of the successor to the consumers,
     // who give it after their wait: a release from here would let a second launch run ahead.)
-    issue(&map_k, 0, n, false, kbar);
-    issue(&map_v, 0, n_early, true, vbar_e);
+    if (!kShared) {
+      issue(&map_k, 0, n, false, kbar);
+      issue(&map_v, 0, n_early, true, vbar_e);
+    }
     bar_sync(1, kDecodeThreads);                         // A: every consumer warp is done with the K slots
     if (kLong && n_late > 0) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // their reads (and a patched row) precede the refill
@@ -697,7 +712,7 @@ static int cluster_capacity(Kernel kernel, int threads, size_t smem, int c, std:
 static int resident_capacity(int device, int c, int tiles) {   // of decode_attn_kernel, `tiles` tiles per CTA
   static std::atomic<int> table[64][kDecodeMaxCluster + 1][kDecodeMaxTiles + 1];
   if (device < 0 || device >= 64 || c < 1 || c > kDecodeMaxCluster || tiles < 0 || tiles > kDecodeMaxTiles) return 0;
-  return cluster_capacity(decode_attn_kernel<true>, kDecodeThreads, decode_smem_bytes(tiles), c, &table[device][c][tiles]);
+  return cluster_capacity(decode_attn_kernel<true, false>, kDecodeThreads, decode_smem_bytes(tiles), c, &table[device][c][tiles]);
 }
 
 static int stream_capacity(int device, int c) {                // of decode_stream_kernel, clusters of c CTAs
@@ -715,16 +730,30 @@ static float with_traffic(float us, int heads, int L) {
 
 cudaError_t decode_setup(DeviceInfo *dev) {
   (void)dev;
-  const cudaError_t e = cudaFuncSetAttribute(decode_attn_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)decode_smem_bytes(kDecodeMaxTiles));
-  if (e != cudaSuccess) return e;
-  const cudaError_t e2 = cudaFuncSetAttribute(decode_attn_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)decode_smem_bytes(kDecodeMaxTiles));
-  if (e2 != cudaSuccess) return e2;
+  for (auto kernel : {decode_attn_kernel<false, false>, decode_attn_kernel<false, true>, decode_attn_kernel<true, false>, decode_attn_kernel<true, true>}) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)decode_smem_bytes(kDecodeMaxTiles));
+    if (e != cudaSuccess) return e;
+  }
   cudaError_t e3 = cudaFuncSetAttribute(decode_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(StShared));
   if (e3 == cudaSuccess) e3 = cudaFuncSetAttribute(decode_stream_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of 16
   if (e3 != cudaSuccess) return e3;
   return cudaFuncSetAttribute(decode_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)decode_tc_smem_bytes(kTcMaxTiles));
+}
+
+// In modes 0 and 1 launches of this many KV heads keep the older, coarser costs of both kernels: with the newer ones 24 x 2561 rows went from
+// 8.5 (whole) to 9.1 us (streamed) and 32 x 1537 from 7.3 to 7.9.
+constexpr int kDecodeManyHeads = 20;
+
+// Whether all nine warps of a CTA ask for its copies, or the ninth alone.  Sharing takes the copies' issue time off the launch, which
+// counts where they are asked for behind the dependency wait, or late because the predecessor's clusters are in the way (us per launch
+// alone / shared: mode 0, 8 heads x 2049 rows 6.5 / 5.0, 1025 rows 4.7 / 4.1; mode 2, 8 x 2049 3.96 / 3.74, 16 x 2049 5.7 / 5.0, 8 x 3000
+// 5.3 / 4.4).  In modes 0 and 1 the eight warps have the query to ask for meanwhile, and few copies are soon asked for by one (8 x
+// 513 3.60 / 3.75, 1 x 4 heads with 7 tiles per CTA 3.61 / 3.75, with 9 3.97 / 3.90; with 64 CTAs and 7 tiles 4.07 / 3.88); nor does it
+// help where V tiles wait for K slots in many CTAs (16 x 3073 8.20 / 8.52), or several clusters per head (8 x 8193 12.0 / 12.4).
+static bool decode_shares_issue(int mode, int ctas, int per_cta, int units, int n_clusters) {
+  if (n_clusters > 1) return false;
+  if (mode == 2) return true;
+  return units < kDecodeManyHeads && per_cta >= (ctas >= 56 ? 7 : 9) && !(2 * per_cta > kDecodeSlots && units >= 12);
 }
 
 // Launch geometry for a reduced cache of L rows: nc clusters of c CTAs per KV head, a CTA taking at most
@@ -734,17 +763,18 @@ cudaError_t decode_setup(DeviceInfo *dev) {
 // computes), which only works if the clusters of two launches fit on the device together, so the cluster sizes
 // are compared by a cost fitted to measurements (below).
 // (15 clusters of 8 whole-SM CTAs fit at once, 22 of 6, 26 of 5, 33 of 4.)
-float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int *n_clusters, int *cs, int *per_cta_tiles,
+float decode_geometry(int L, int heads, const DeviceInfo *dev, int mode, int *n_clusters, int *cs, int *per_cta_tiles,
                       int *smem_bytes) {
   const int n_tiles = (L + 15) / 16;
   int c = 1;
   while (c < kDecodeBaseCluster && c * 2 <= n_tiles) c <<= 1;                   // cluster size 1, 2, 4 or 8
   int nc = (n_tiles + c * kDecodeMaxTiles - 1) / (c * kDecodeMaxTiles);          // the fewest clusters per head
   float best = 0.f;
+  const bool many = mode != 2 && heads >= kDecodeManyHeads;
   int best_waves = 1;
-  bool apart = false;                                    // two launches' clusters do not fit on the device together
   if (dev != nullptr && heads > 0) {
     int best_c = c, best_nc = nc;
+    const float bytes = (float)heads * (float)L * (4.f * kHeadDim);
     // up to kDecodeExtraClusters more clusters per head than needed: beyond one cluster the results are merged
     // through scratch anyway, and more, smaller clusters leave fewer V tiles waiting for a K slot
     for (int n_try = nc; n_try <= (nc > 1 ? nc + kDecodeExtraClusters : nc); ++n_try) {
@@ -753,19 +783,38 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int
         if (per > kDecodeMaxTiles) continue;
         const int cap = resident_capacity(dev->device, cand, per);
         if (cap <= 0) continue;
-        // measured on this part (us per launch, batch 1 x 8 heads, L = 1025 / 2049 / 4097, clusters of 5 to 8):
-        // 2.97 + 0.0445 per tile of a CTA; the same again per tile when the clusters of two launches do not fit
-        // together (the copies are then issued on the critical path); 0.084 per V tile that has to wait for a K
-        // slot; 3.4 for the merge through scratch (L = 8193, 1 and 8 heads)
-        const int late = 2 * per > kDecodeSlots ? 2 * per - kDecodeSlots : 0;
-        const int waves = (heads * n_try + cap - 1) / cap;                      // of one launch
-        const float one = 2.97f + 0.0445f * (float)per * (2 * heads * n_try <= cap ? 1.f : 2.f) + 0.084f * (float)late +
-                          (n_try > 1 ? 3.4f : 0.f);
-        const float cost = (float)waves * one;
-        if (best == 0.f || cost < best) {
-          best = cost; best_c = cand; best_nc = n_try; best_waves = waves;
-          apart = 2 * heads * n_try > cap;
+        // Fitted to every cluster size (4 to 8) at 1 to 48 heads x 129 .. 4097 rows in all overlap modes, G = 4 (us per launch): a time
+        // per tile of a CTA, 0.3 - 0.5 and a time per V tile that waits for a K slot where some do, more where the clusters of
+        // two launches do not fit on the device together, up to as much again as they overfill it; and beside that what moving
+        // the rows takes.  3.4 for the merge through scratch (L = 8193, 1 and 8 heads).  (What these rules choose is on average
+        // 0.2 % slower than the best cluster size or streamed launch of each case in mode 2, 0.9 % in mode 0, 1.3 % in mode 1.)
+        const int late = 2 * per > kDecodeSlots ? 2 * per - kDecodeSlots : 0, units = heads * n_try;
+        const int waves = (units + cap - 1) / cap;                              // of one launch
+        const bool is_long = per > kQkGroup * kDecodeWarps;
+        const float over = 2 * units > cap ? (float)((units < cap ? 2 * units : 2 * cap) - cap) / (float)cap : -1.f;
+        const float share = (float)n_tiles / (float)(cand * n_try);
+        float one, cost;
+        if (many) {
+          one = 2.97f + 0.0445f * (float)per * (2 * units <= cap ? 1.f : 2.f) + 0.084f * (float)late;
+        } else if (mode == 2) {
+          one = 2.89f + 0.035f * (float)per + (is_long ? 0.26f + 0.056f * (float)late : 0.f) + (over >= 0.f ? 0.31f + 0.59f * over : 0.f);
+        } else {
+          one = decode_shares_issue(mode, units * cand, per, units, n_try) ? 3.11f + 0.073f * share + (is_long ? 0.49f + 0.04f * (float)late : 0.f)
+                                                                           : 3.f + 0.057f * share + 0.072f * (share > 6.f ? share - 6.f : 0.f);
+          one += over >= 0.f ? 0.21f + 0.28f * over : 0.f;
         }
+        if (n_try > 1) one += 3.4f;
+        one = (float)waves * one + (many ? 0.f : 0.5f * (float)(waves - 1));
+        if (many) {
+          cost = one;
+        } else if (mode == 2) {
+          const float t = 1.f + bytes / 5.3e6f;
+          cost = powf(powf(one, 2.9f) + powf(t, 2.9f), 1.f / 2.9f);
+        } else {
+          const float t = 1.f + bytes / 7.3e6f;
+          cost = sqrtf(one * one + t * t);
+        }
+        if (best == 0.f || cost < best) { best = cost; best_c = cand; best_nc = n_try; best_waves = waves; }
       }
     }
     c = best_c;
@@ -778,25 +827,22 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, bool overlap, int
   *cs = c;
   *per_cta_tiles = per_cta;
   *smem_bytes = (int)decode_smem_bytes(per_cta);
-  // without overlap: 3.9 + 0.14 per tile (the copies are issued on the critical path: L = 257 .. 4097, 1 to 16 heads)
-  if (best > 0.f && !overlap) best = (float)best_waves * (3.9f + 0.14f * (float)per_cta + (nc > 1 ? 3.4f : 0.f));
-  // (against the streamed launch: 16 / 24 / 32 heads x 2049 rows 5.9 / 7.7 / 8.5)
-  if (best > 0.f && overlap && apart) best += 0.027f * (float)(best_waves * per_cta);
-  return best > 0.f ? with_traffic(best, heads, L) : 0.f;
+  if (many && best > 0.f) best = with_traffic((float)best_waves * (3.9f + 0.14f * (float)per_cta + (nc > 1 ? 3.4f : 0.f)), heads, L);
+  return best;
 }
 
-// The best launch of decode_stream_kernel: CTAs per head, heads per CTA, and its cost in us (0: none).  Fitted to forced launches
-// of every split, 1 to 128 heads x 125 .. 8193 rows x 1 to 8 query heads per KV head (G).  Overlapping: 1.75 plus 0.017 per CTA of a
+// The best launch of decode_stream_kernel: CTAs per head, heads per CTA, and its cost in us (0: none).  Mode 2, fitted to forced launches
+// of every split, 1 to 128 heads x 125 .. 8193 rows x 1 to 8 query heads per KV head (G): 1.75 plus 0.017 per CTA of a
 // cluster, 0.47 per tile of a warp (the ring's three tiles per warp in flight against the latency of a copy; 0.6 where a CTA takes
 // whole heads), 0.06 per query head, 0.41 per round of the finishing stage (a thread takes two columns of a head: a cluster of 2 with
 // G = 8 needs two), 0.8 per further head of a CTA; up to 1.1 more when two launches' CTAs do not fit on the device together.  A second
-// wave costs a whole time again.  Not overlapping: 3.9, 0.025, 0.6 and 0.8 in place of these, 1 % per query head beyond four.
-// (Without the terms in G, launches with 7 or 8 query heads were streamed where bringing the cache in whole is faster: us whole /
-// streamed at 16 heads x 1537 rows, G = 8: 4.27 / 4.66, 16 x 765 3.64 / 4.04, 4 x 125 2.94 / 3.26.  Of 1173 launches of that sweep in
-// all overlap modes 49 took over 1.5 % longer than before there were streamed ones, now 27; the mean of all 0.787 of the time, now 0.784.)
-static float stream_geometry(int L, int heads, int G, const DeviceInfo &dev, bool overlap, int *split, int *per_cta) {
+// wave costs a whole time again.  Modes 0 and 1, fitted against the resident kernel as it is now (1 to 48 heads x 129 .. 4097 rows):
+// 3.47 and 2.69, 0.52 and 0.62 per tile of a warp, 1 % per query head beyond four.
+static float stream_geometry(int L, int heads, int G, const DeviceInfo &dev, int mode, int *split, int *per_cta) {
   const int n_tiles = (L + 15) / 16;
   if ((int64_t)n_tiles * heads > (int64_t)1 << 30) return 0.f;
+  const bool overlap = mode == 2, many = heads >= kDecodeManyHeads;
+  const float base = many ? 3.9f : (mode == 0 ? 3.47f : 2.69f), per_s = many ? 0.025f : 0.006f, per_round = many ? 0.6f : (mode == 0 ? 0.52f : 0.62f);
   float best = 0.f;
   for (int s = 1; s <= kStMaxCluster && s <= n_tiles; s <<= 1) {
     const int cap = s == 1 ? kStreamCtasPerSm * dev.n_sm : s * stream_capacity(dev.device, s);
@@ -807,7 +853,8 @@ static float stream_geometry(int L, int heads, int G, const DeviceInfo &dev, boo
     const int rounds = (per * ((n_tiles + s - 1) / s) + kStWarps - 1) / kStWarps;
     const int finish = s == 1 ? 0 : (G * (kHeadDim / 2) + s * kStThreads - 1) / (s * kStThreads);   // (s == 1: no such stage)
     const float one = overlap ? 1.75f + 0.017f * (float)s + (s > 1 ? 0.47f : 0.6f) * (float)rounds + 0.06f * (float)G + 0.41f * (float)finish + 0.8f * (float)(per - 1)
-                              : (3.9f + 0.025f * (float)s + 0.6f * (float)rounds + 0.8f * (float)(per - 1)) * (1.f + 0.01f * (float)(G > 4 ? G - 4 : 0));
+                              : (base + per_s * (float)s + per_round * (float)rounds + 0.8f * (float)(per - 1)) *
+                                    (1.f + 0.01f * (float)(G > 4 ? G - 4 : 0));
     float cost = with_traffic((float)waves * one, heads, L);
     if (2 * ctas > cap) cost += (overlap ? 0.13f : 0.3f) + (overlap ? 0.95f : 1.2f) * (float)(2 * (ctas < cap ? ctas : cap) - cap) / (float)cap;
     if (best == 0.f || cost < best) { best = cost; *split = s; *per_cta = per; }
@@ -851,13 +898,13 @@ static bool make_cache_map(CUtensorMap *map, const uint16_t *base, const DecodeP
 
 cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStream_t stream) {
   int n_clusters, cs, per_cta, smem, split = 1, heads_per_cta = 1;
-  const bool overlap = p.overlapping;
-  const float cost = decode_geometry(p.L, p.B * p.H_kv, &dev, overlap, &n_clusters, &cs, &per_cta, &smem);
+  const int mode = p.overlapping ? 2 : p.pdl_mode;
+  const float cost = decode_geometry(p.L, p.B * p.H_kv, &dev, mode, &n_clusters, &cs, &per_cta, &smem);
   const bool tc = p.variant == 2 && n_clusters == 1 && per_cta <= kTcMaxTiles;
   // Caches that fill the SMs more than once, and long ones, are streamed; short ones are brought in whole.  (us per
   // launch whole / streamed, overlapping: 8 heads x 2049 rows 4.1 / 4.7, 8 x 8193 11.0 / 9.4, 64 x 2049 17.4 / 13.4,
   // 256 x 2049 84.8 / 42.8)
-  const float stream_cost = tc ? 0.f : stream_geometry(p.L, p.B * p.H_kv, p.G, dev, overlap, &split, &heads_per_cta);
+  const float stream_cost = tc ? 0.f : stream_geometry(p.L, p.B * p.H_kv, p.G, dev, mode, &split, &heads_per_cta);
   const bool streamed = stream_cost > 0.f && cost > 0.f && stream_cost < cost;
   CUtensorMap map_k, map_v;
   if (!make_cache_map(&map_k, p.Kc, p) || !make_cache_map(&map_v, p.Vc, p)) return cudaErrorInvalidValue;
@@ -889,8 +936,10 @@ cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStre
   }
   // the short instance keeps three tiles' scores per warp and has every V tile resident from the start
   const bool is_long = 2 * per_cta > kDecodeSlots || per_cta > kQkGroup * kDecodeWarps;
-  return is_long ? cudaLaunchKernelEx(&cfg, decode_attn_kernel<true>, p, map_k, map_v, decode_slots(per_cta))
-                 : cudaLaunchKernelEx(&cfg, decode_attn_kernel<false>, p, map_k, map_v, decode_slots(per_cta));
+  const bool shared = decode_shares_issue(mode, (int)(cfg.gridDim.x * cfg.gridDim.y * cfg.gridDim.z), per_cta, p.B * p.H_kv * n_clusters, n_clusters);
+  const auto kernel = is_long ? (shared ? decode_attn_kernel<true, true> : decode_attn_kernel<true, false>)
+                              : (shared ? decode_attn_kernel<false, true> : decode_attn_kernel<false, false>);
+  return cudaLaunchKernelEx(&cfg, kernel, p, map_k, map_v, decode_slots(per_cta));
 }
 
 }  // namespace sagekv
