@@ -46,3 +46,15 @@ def hint_of(rows, E):
         out[h, :512] = np.bincount(bins, minlength=512).astype(np.uint32)
         out[h, 512:] = [0x53414745, E, bin0, kmax]
     return out
+
+
+def kernels_of(f):
+    """Names of the kernels that f() launches, in order, demangled, without return type, namespace and parameters."""
+    from torch.profiler import ProfilerActivity, profile
+    f()                                                           # (what is loaded on first use)
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        f()
+        torch.cuda.synchronize()
+    names = [(e.time_range.start, e.name) for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA]
+    return [n.split("sagekv::")[1].split("(")[0] for _, n in sorted(names) if "sagekv::" in n]

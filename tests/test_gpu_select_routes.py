@@ -1,0 +1,76 @@
+"""Which kernel a selection takes, on both sides of every line of the rule for rows of 8193 to 16384 scores: few and many kept scores,
+up to and beyond one CTA per SM, with and without a gather, many static rows beside it, a histogram behind the rows.  The lines are
+where one way became slower than the other when measured; results are the same, bit-exact against the oracle."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import sagekv_oracle as O
+from helpers import bits, kernels_of
+
+pytestmark = pytest.mark.gpu
+
+SHORT, CLUSTER, GENERAL = "select_short_kernel", "select_compact_kernel", "select_general_kernel"
+
+
+def select(rows, E, k, S, R, G, hint, gather, kernel):
+    from paper_2503_08879_b200 import binding as B
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    H = {"half": n_sm // 2, "one": n_sm, "more": n_sm + 8, "5/4": 5 * n_sm // 4 + 8, "two": 2 * n_sm, "three": 3 * n_sm, "3+": 3 * n_sm + 8}.get(rows, rows)
+    H -= H % G
+    Hkv, N = H // G, S + E + R + 1
+    gen = torch.Generator(device="cuda").manual_seed(E + k)
+    sk = B.SageKV(H, Hkv, 128, 1, max_ctx=N, max_len=S + G * k + R + 1)
+    sk.set_select_hint(hint)
+    scores = torch.exp(1.5 * torch.randn(H, sk.score_stride(N, S, R), generator=gen, device="cuda") - 12)
+    if gather:
+        K = torch.randint(-9999, 9999, (1, 1, N, 128), generator=gen, device="cuda", dtype=torch.int16).view(torch.bfloat16).expand(1, Hkv, N, 128)
+        cache = sk.new_layer(S, R, G * k)
+        names = kernels_of(lambda: sk.select_compact(scores, K, K, S, R, G * k, cache))
+        idx = cache.indices()[0]
+    else:
+        idx = torch.full((1, H, k), -1, dtype=torch.int32, device="cuda")
+        names = kernels_of(lambda: B.sagekv_select_topk(sk.ctx, scores, scores.stride(0), E, k, idx))
+        idx = idx[0] + S
+    assert sk.status() == 0
+    assert names[-1].startswith(kernel) and names[:-1] in ([], ["copy_static_kernel"]), names
+    some = sorted({0, H // 2, H - 1})
+    want = O.select(scores[some, :E].cpu().numpy(), k, S)
+    assert np.array_equal(idx[some].cpu().numpy(), want)
+    if gather:
+        for i, h in enumerate(some):
+            j = S + h % G * k
+            assert np.array_equal(bits(cache.Kc[0, h // G, j:j + k]), bits(K[0, 0])[want[i]])
+        last = torch.cat([K[0, 0, :S], K[0, 0, S + E:]])
+        got = torch.cat([cache.Vc[0, -1, :S], cache.Vc[0, -1, S + G * k:cache.state.len]])
+        assert torch.equal(got.view(torch.int16), last.view(torch.int16))
+    sk.close()
+    return names
+
+
+@pytest.mark.parametrize("rows,E,k,kernel", [
+    (640, 8192, 256, SHORT), ("one", 8193, 256, SHORT), ("more", 8193, 256, CLUSTER), ("one", 16384, 40, SHORT), ("more", 16384, 40, CLUSTER),
+    ("half", 16384, 512, SHORT), ("one", 16384, 384, SHORT), ("one", 16384, 385, CLUSTER), ("more", 16384, 257, SHORT), ("5/4", 9000, 257, CLUSTER),
+    ("5/4", 9000, 512, CLUSTER), ("5/4", 16384, 513, SHORT), (32, 16385, 512, SHORT), ("one", 16385, 64, CLUSTER), (16, 33000, 2049, GENERAL)])
+def test_with_a_gather(rows, E, k, kernel):
+    select(rows, E, k, 3, 20, 4, 0, True, kernel)
+
+
+@pytest.mark.parametrize("rows,E,k,kernel", [
+    ("more", 14336, 256, SHORT), ("two", 14336, 256, SHORT), ("two", 14337, 256, CLUSTER), ("three", 16384, 256, SHORT), ("3+", 9000, 256, CLUSTER),
+    ("3+", 9000, 257, SHORT)])
+def test_without_a_gather(rows, E, k, kernel):
+    select(rows, E, k, 0, 20, 1, 0, False, kernel)
+
+
+@pytest.mark.parametrize("rows,S,R,k,kernel", [(80, 1999, 2000, 256, SHORT), (80, 2000, 2000, 256, CLUSTER), (80, 2000, 2000, 513, SHORT)])
+def test_many_static_rows(rows, S, R, k, kernel):
+    names = select(rows, 9000, k, S, R, 4, 0, True, kernel)
+    assert names[0] == "copy_static_kernel"
+
+
+@pytest.mark.parametrize("rows,E,k,kernel", [("half", 14337, 1500, SHORT), ("one", 14337, 128, SHORT), ("one", 16384, 129, CLUSTER), ("more", 16384, 40, CLUSTER),
+                                             ("more", 14337, 600, CLUSTER), (16, 16385, 40, CLUSTER)])
+def test_with_a_histogram_behind_the_rows(rows, E, k, kernel):
+    select(rows, E, k, 3, 20, 4, 1, True, kernel)
