@@ -396,14 +396,19 @@ static ShortPlan short_plan(const SelectParams &p, int n_sm) {
 
 // Which rows: up to 8192 scores all (us per launch, clusters that exchange / this: 32 rows of 3963, k_q = 64, 10.0 / 5.2, k_q = 1024
 // with as many sink and recent rows 24.6 / 13.2; 32 x 8184, k_q = 29, indices only, 9.6 / 5.3; 1024 x 8184, k_q = 240, 84 / 72).
-// Up to 16384, where a CTA has its SM to itself: all that a cluster would need four CTAs or more for (k_q > 512: 512 x 16384, k_q =
-// 600, 129 / 100), and of the others those that are one wave, where two clusters of one CTA share an SM (k_q = 240, with the gather: 32
-// rows 11.0 / 8.3, 128 16.8 / 15.1, 160 21.2 / 23.3, 256 25.7 / 32.0, 1024 82 / 107).  More closely, a row's CTA alone takes longer over
-// 400 rows of K and V than two (128 rows, k_q = 400 19.6 / 20.3, 512 22.7 / 23.8) unless the clusters of two just miss their wave (152, k_q =
-// 400, 32.3 / 30.5; 200 35.3 / 39.3); without a gather it is ahead for longer (160 rows, k_q = 256, 12.8 / 12.4, 256 x 12500 13.5 / 12.8, 256 x
-// 16384 13.4 / 14.1, 400 21.3 / 21.5, 1024 43.4 / 47.2); behind very many static rows it leaves the copies less room (96 rows, k_q = 256,
-// 98328 static rows 25.7 / 27.4; 64, 65552 19.7 / 19.3).  With a histogram behind the rows a cluster saves its exchanges: 64 rows, k_q = 479,
-// 15.2 / 13.1, but 128 21.6 / 24.6; 128 with k_q = 128 13.2 / 12.5; 256 with k_q = 64 16.4 / 22.1.
+// Up to 16384, where a CTA has its SM to itself (k_q = kept scores):
+//  - those that clusters would need four CTAs or more for, all (512 rows x 16384, k_q = 600, 129 / 100);
+//  - those for two CTAs, where this kernel copies the static rows along (128 rows x 16384, k_q = 400, 19.2 / 16.3; 512 rows, k_q = 512, 81.5 / 73.4).  With a
+//    kernel of their own for these, which clusters with twice the warps may do without, a CTA's turn over 400 rows of K and V shows: 76 rows,
+//    k_q = 512, 20.0 / 19.1, 128 22.7 / 23.8, 196, k_q = 400, 33.7 / 37.3; but 128 rows, k_q = 300, 17.1 / 16.8, with more static rows than kept ones,
+//    k_q = 512, 25.8 / 24.4, and between one wave of these and two of such clusters, 152 rows, k_q = 400, 32.3 / 30.5 (where those need the kernel
+//    too 33.6 / 35.3);
+//  - those for one, two of which share an SM, up to one row per SM (k_q = 240: 32 rows 11.0 / 8.3, 128 16.8 / 15.1, 160 21.2 / 23.3, 256 25.7 /
+//    32.0, 1024 82 / 107); without a gather longer (160 rows, k_q = 256, 12.8 / 12.4, 256 x 12500 13.5 / 12.8, 256 x 16384 13.4 / 14.1, 400 21.3 /
+//    21.5, 1024 43.4 / 47.2);
+//  - not behind very many static rows, for whose copies it leaves less room (96 rows, k_q = 256, 98328 of them 25.7 / 27.4; 64, 65552 19.7 / 19.3);
+//  - with a histogram behind the rows, which saves a cluster its exchanges: 64 rows, k_q = 479, 15.2 / 13.1, but 128 21.6 / 24.6; 128 with
+//    k_q = 128 13.2 / 12.5; 256 with k_q = 64 16.4 / 22.1.
 // Longer ones, where a thread has 64 scores, up to two rows for three SMs, and where
 // nothing has to be copied beside: 32 x 25236, k_q = 479, 12.2 / 11.2; 84 x 25236 19.5 / 16.3; but 128 x 25236 20.3 / 21.9, and with 2049
 // static rows 32 x 25236, k_q = 512, 14.3 / 15.7.
@@ -420,7 +425,9 @@ static bool short_rows_apply(const SelectParams &p, int n_sm, bool sketch) {
   if (p.Kc == nullptr)
     return 2 * p.k_q > kSelThreads || (rows <= 3 * (int64_t)n_sm && !(2 * rows > 3 * (int64_t)n_sm && rows <= 2 * (int64_t)n_sm && p.E > 7 * 4 * kSelThreads));
   if (2 * p.k_q <= kSelThreads) return rows <= n_sm;
-  return 2 * rows <= n_sm || (rows <= n_sm ? plan.beside || 4 * p.k_q <= 3 * kSelThreads : 4 * rows <= 5 * (int64_t)n_sm);
+  if (!plan.beside) return true;
+  if (rows <= n_sm) return 3 * rows <= 2 * (int64_t)n_sm || 4 * p.k_q <= 3 * kSelThreads || p.S + p.R >= p.k_q;
+  return 10 * rows <= 13 * (int64_t)n_sm && p.S + p.R < kStaticPerWarp * p.G * 2 * kSelWarps;
 }
 
 static cudaError_t launch_select_short(const SelectParams &p, int n_sm, cudaStream_t stream) {

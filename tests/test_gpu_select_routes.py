@@ -1,6 +1,6 @@
 """Which kernel a selection takes, on both sides of every line of the rule for rows of 8193 to 16384 scores: few and many kept scores,
-up to and beyond one CTA per SM, with and without a gather, many static rows beside it, a histogram behind the rows.  The lines are
-where one way became slower than the other when measured; results are the same, bit-exact against the oracle."""
+up to and beyond one CTA per SM, with and without a gather, many static rows beside it, a histogram behind the rows.  The lines are where one
+way became slower than the other when measured; results are the same, bit-exact against the oracle."""
 
 import numpy as np
 import pytest
@@ -17,7 +17,7 @@ SHORT, CLUSTER, GENERAL = "select_short_kernel", "select_compact_kernel", "selec
 def select(rows, E, k, S, R, G, hint, gather, kernel):
     from paper_2503_08879_b200 import binding as B
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
-    H = {"half": n_sm // 2, "one": n_sm, "more": n_sm + 8, "5/4": 5 * n_sm // 4 + 8, "two": 2 * n_sm, "three": 3 * n_sm, "3+": 3 * n_sm + 8}.get(rows, rows)
+    H = {"half": n_sm // 2, "one": n_sm, "more": n_sm + 8, "13/10": 13 * n_sm // 10 + 4, "two": 2 * n_sm, "three": 3 * n_sm, "3+": 3 * n_sm + 8}.get(rows, rows)
     H -= H % G
     Hkv, N = H // G, S + E + R + 1
     gen = torch.Generator(device="cuda").manual_seed(E + k)
@@ -49,12 +49,14 @@ def select(rows, E, k, S, R, G, hint, gather, kernel):
     return names
 
 
-@pytest.mark.parametrize("rows,E,k,kernel", [
-    (640, 8192, 256, SHORT), ("one", 8193, 256, SHORT), ("more", 8193, 256, CLUSTER), ("one", 16384, 40, SHORT), ("more", 16384, 40, CLUSTER),
-    ("half", 16384, 512, SHORT), ("one", 16384, 384, SHORT), ("one", 16384, 385, CLUSTER), ("more", 16384, 257, SHORT), ("5/4", 9000, 257, CLUSTER),
-    ("5/4", 9000, 512, CLUSTER), ("5/4", 16384, 513, SHORT), (32, 16385, 512, SHORT), ("one", 16385, 64, CLUSTER), (16, 33000, 2049, GENERAL)])
-def test_with_a_gather(rows, E, k, kernel):
-    select(rows, E, k, 3, 20, 4, 0, True, kernel)
+@pytest.mark.parametrize("rows,E,k,R,kernel", [
+    (640, 8192, 256, 20, SHORT), ("one", 8193, 256, 20, SHORT), ("more", 8193, 256, 20, CLUSTER), ("one", 16384, 40, 20, SHORT),
+    ("more", 16384, 40, 20, CLUSTER), ("half", 16384, 512, 20, SHORT), ("more", 16384, 257, 20, SHORT), (400, 8193, 512, 124, SHORT),
+    ("one", 16384, 384, 125, SHORT), ("one", 16384, 385, 125, CLUSTER), (96, 16384, 512, 125, SHORT), (112, 16384, 512, 125, CLUSTER),
+    (192, 16384, 512, 125, SHORT), ("13/10", 9000, 257, 125, CLUSTER), ("13/10", 9000, 512, 125, CLUSTER), ("13/10", 16384, 513, 125, SHORT),
+    (32, 16385, 512, 20, SHORT), ("one", 16385, 64, 20, CLUSTER), (16, 33000, 2049, 20, GENERAL)])
+def test_with_a_gather(rows, E, k, R, kernel):               # 3 + R + 1 static rows: 128 are copied along by one CTA per row
+    select(rows, E, k, 3, R, 4, 0, True, kernel)
 
 
 @pytest.mark.parametrize("rows,E,k,kernel", [
@@ -64,10 +66,11 @@ def test_without_a_gather(rows, E, k, kernel):
     select(rows, E, k, 0, 20, 1, 0, False, kernel)
 
 
-@pytest.mark.parametrize("rows,S,R,k,kernel", [(80, 1999, 2000, 256, SHORT), (80, 2000, 2000, 256, CLUSTER), (80, 2000, 2000, 513, SHORT)])
+@pytest.mark.parametrize("rows,S,R,k,kernel", [(80, 1999, 2000, 256, SHORT), (80, 2000, 2000, 256, CLUSTER), (80, 2000, 2000, 513, SHORT),
+                                                     (112, 300, 300, 512, SHORT), (160, 64, 191, 300, SHORT), (160, 64, 192, 300, CLUSTER)])
 def test_many_static_rows(rows, S, R, k, kernel):
     names = select(rows, 9000, k, S, R, 4, 0, True, kernel)
-    assert names[0] == "copy_static_kernel"
+    assert names[0] == "copy_static_kernel", names
 
 
 @pytest.mark.parametrize("rows,E,k,kernel", [("half", 14337, 1500, SHORT), ("one", 14337, 128, SHORT), ("one", 16384, 129, CLUSTER), ("more", 16384, 40, CLUSTER),
