@@ -1192,7 +1192,11 @@ __device__ __forceinline__ void general_select_wide(cg::cluster_group &cluster, 
   cluster.sync();   // no CTA moves on (and may exit) while a peer still reads its shared memory
 }
 
-__global__ void __launch_bounds__(kSelThreads, 2) select_general_kernel(const SelectParams p, int behind_static, int chunk, int resident, int list_cap) {
+// kRoom: the instance for launches whose static rows are copied beside them by a kernel that needs room on the same SMs (bound as
+// select_compact_kernel<false> is: 56 registers; see launch_select_compact for when).
+template <bool kRoom>
+__global__ void __launch_bounds__(kRoom ? kSelThreads + 64 : kSelThreads, 2)
+    select_general_kernel(const SelectParams p, int behind_static, int chunk, int resident, int list_cap) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cg::cluster_group cluster = cg::this_cluster();
   cluster.barrier_arrive();   // every CTA of the cluster runs before anyone writes into a peer
@@ -1384,7 +1388,9 @@ cudaError_t select_compact_setup() {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(select_compact_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(select_general_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
+  e = cudaFuncSetAttribute(select_general_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(select_general_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelSmemLimit);
   if (e != cudaSuccess) return e;
   e = select_short_setup();
   if (e != cudaSuccess) return e;
@@ -1471,8 +1477,16 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   }
   const int64_t sketch_off = try_fast && sketch && !list ? sketch_offset(p.E) : (int64_t)-1;
   const int64_t list_off = try_fast && list ? sketch_offset(p.E) : (int64_t)-1;
-  if (!try_fast)
-    return launch_next(select_general_kernel, dim3((unsigned)(n_rows * cs)), kSelThreads, smem, stream, cs, pl, (int)beside, chunk, (int)resident, list_cap);
+  if (!try_fast) {
+    // Two CTAs of 64 registers a thread leave an SM none for the static rows' kernel.  Where two share an SM with shared memory left
+    // for that kernel, and the rows to be copied beside are at least half as many as the selected ones, the room is worth more than the
+    // registers (us per launch with 64 / 56: 32 pooled rows x 50000, k_q = 2100, 4097 static rows 72.5 / 55.6, 64 x 17000, 8000, 202 / 177; but
+    // 2048 static rows beside k_q = 8000 157 / 162, 16 rows x 17000, k_q = 4096 45.4 / 46.8, 8 rows 31.0 / 33.6, 32 x 100000 82.2 / 84.7).
+    const bool room = beside && (int64_t)n_rows * cs > n_sm && 2 * (smem + 1024) + kStaticSmem + 1024 <= (size_t)kSelSmemLimit + 1024 &&
+                      2 * (int64_t)n_static >= (int64_t)p.G * p.k_q;
+    return launch_next(room ? select_general_kernel<true> : select_general_kernel<false>, dim3((unsigned)(n_rows * cs)), kSelThreads, smem, stream,
+                       cs, pl, (int)beside, chunk, (int)resident, list_cap);
+  }
   return launch_next(ahead ? select_compact_kernel<true> : select_compact_kernel<false>, dim3((unsigned)(n_rows * cs)), kSelThreads, smem,
                      stream, cs, pl, (int)beside, chunk, (int)resident, list_cap, cand_cap, sketch_off, list_off);
 }

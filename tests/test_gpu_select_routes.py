@@ -1,6 +1,7 @@
 """Which kernel a selection takes, on both sides of every line of the rule for rows of 8193 to 16384 scores: few and many kept scores,
-up to and beyond one CTA per SM, with and without a gather, many static rows beside it, a histogram behind the rows.  The lines are where one
-way became slower than the other when measured; results are the same, bit-exact against the oracle."""
+up to and beyond one CTA per SM, with and without a gather, many static rows beside it, a histogram behind the rows; and of that for the
+large selections' instance that leaves room for the static rows' kernel.  The lines are where one way became slower than the other when
+measured; results are the same, bit-exact against the oracle."""
 
 import numpy as np
 import pytest
@@ -77,3 +78,11 @@ def test_many_static_rows(rows, S, R, k, kernel):
                                              ("more", 14337, 600, CLUSTER), (16, 16385, 40, CLUSTER)])
 def test_with_a_histogram_behind_the_rows(rows, E, k, kernel):
     select(rows, E, k, 3, 20, 4, 1, True, kernel)
+
+
+@pytest.mark.parametrize("rows,E,k,S,R,kernel", [
+    (32, 17000, 8192, 2048, 2047, GENERAL + "<true>"), (32, 17000, 8193, 2048, 2047, GENERAL + "<false>"), (32, 50002, 2100, 600, 449, GENERAL + "<true>"),
+    (32, 60002, 4300, 2048, 2048, GENERAL + "<false>"),
+    (8, 50002, 2100, 2048, 2048, GENERAL + "<false>"), (32, 100001, 4096, 2048, 2048, GENERAL + "<false>"), (32, 50002, 2100, 4, 20, GENERAL + "<false>")])
+def test_large_selections_beside_static_rows(rows, E, k, S, R, kernel):
+    select(rows, E, k, S, R, 1, 0, True, kernel)
