@@ -218,7 +218,9 @@ __global__ void __launch_bounds__(kSelThreads + 64, kVec > 4 ? 1 : 2)
         while (m) {
           const int pos = 4 * (v0 + u * 32) + __ffs(m) - 1;
           m &= m - 1;
-          cand[at++] = ((unsigned long long)score_key(grow[pos]) << 32) | (0xffffffffu - (uint32_t)pos);   // (an L1 hit)
+          if (SAGEKV_OK_INDEX(p.status, pos < p.E && at < cand_cap))
+            cand[at] = ((unsigned long long)score_key(grow[pos]) << 32) | (0xffffffffu - (uint32_t)pos);   // (an L1 hit)
+          ++at;
         }
       }
       __syncthreads();

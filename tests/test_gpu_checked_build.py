@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 FILES = ["tests/test_gpu_score_fuzz.py", "tests/test_gpu_select_fuzz.py", "tests/test_gpu_decode_fuzz.py",
          "tests/test_gpu_select_and_errors.py", "tests/test_gpu_refresh.py", "tests/test_gpu_decode_stream.py",
-         "tests/test_gpu_select_static.py", "tests/test_gpu_select_limits.py", "tests/test_gpu_checked_static.py"]
+         "tests/test_gpu_select_static.py", "tests/test_gpu_select_limits.py", "tests/test_gpu_checked_static.py",
+         "tests/test_gpu_select_short.py", "tests/test_gpu_select_general.py", "tests/test_gpu_decode_issue.py"]
 PARITY = "tests/test_gpu_parity.py"
 PARITY_CASES = "c1_full or scaled or strided or group_sizes or degenerate or softmax_scale or dependent or prefetch"
 
