@@ -1,6 +1,6 @@
 """What a call finds when the kernel directly before it on the stream has written its inputs, where the selection reads them
-while its own static rows are copied by a kernel beside it; alone, and with calls of another context put on the same stream
-from a second thread, between a call's launches too.  And a decode that reads its cache ahead, behind two select calls that
+while its own static rows are copied by a kernel beside it (by clusters, and by single CTAs); alone, and with calls of another
+context put on the same stream from a second thread, between a call's launches too.  And a decode that reads its cache ahead, behind two select calls that
 run ahead.  Bit-exact against the same calls one at a time."""
 
 import threading
@@ -8,10 +8,12 @@ import threading
 import pytest
 import torch
 
+from helpers import kernels_of
+
 pytestmark = pytest.mark.gpu
 
-Bt, Hkv, G, E, k_q, S, R = 2, 4, 4, 25001, 300, 600, 3000        # 3601 static rows per head: copied beside the selection
-H, N = Hkv * G, S + E + R + 1
+Bt, Hkv, G, k_q, S, R = 2, 4, 4, 300, 600, 3000                  # 3601 static rows per head: copied beside the selection
+H = Hkv * G
 
 
 @pytest.fixture(scope="module")
@@ -20,16 +22,17 @@ def B():
     return binding
 
 
-def inputs(gen):
+def inputs(gen, E):
+    N = S + E + R + 1
     rnd = lambda *s: torch.randn(*s, generator=gen, device="cuda").to(torch.bfloat16)
     return rnd(Bt, Hkv, N, 128), rnd(Bt, Hkv, N, 128), torch.rand(Bt * H, (E + 3) // 4 * 4, generator=gen, device="cuda")
 
 
 class Selection:
-    def __init__(self, B, seed):
+    def __init__(self, B, seed, E, kernel):
         gen = torch.Generator(device="cuda").manual_seed(seed)
-        self.sets = [inputs(gen) for _ in range(3)]
-        self.sk = B.SageKV(H, Hkv, 128, Bt, max_ctx=N, max_len=S + G * k_q + R + 1)
+        self.sets = [inputs(gen, E) for _ in range(3)]
+        self.sk = B.SageKV(H, Hkv, 128, Bt, max_ctx=S + E + R + 1, max_len=S + G * k_q + R + 1)
         self.now = [torch.empty_like(x) for x in self.sets[0]]
         self.cache = self.sk.new_layer(S, R, G * k_q)
         self.want = []
@@ -39,6 +42,8 @@ class Selection:
             self.select()
             torch.cuda.synchronize()
             self.want.append([x.clone() for x in (self.cache.idx, self.cache.Kc, self.cache.Vc)])
+        names = kernels_of(self.select)
+        assert names[0] == "copy_static_kernel" and names[1].startswith(kernel) and len(names) == 2, names
 
     def write(self, i):
         for x, y in zip(self.now, self.sets[i]):
@@ -58,16 +63,21 @@ class Selection:
                 x.zero_()
 
 
-def test_inputs_written_directly_before(B):
-    s, bad = Selection(B, 1), torch.zeros((), dtype=torch.int64, device="cuda")
+ROWS = pytest.mark.parametrize("E,kernel", [(25001, "select_compact_kernel"), (12001, "select_short_kernel"), (3001, "select_short_kernel")])
+
+
+@ROWS
+def test_inputs_written_directly_before(B, E, kernel):
+    s, bad = Selection(B, 1, E, kernel), torch.zeros((), dtype=torch.int64, device="cuda")
     s.rounds(60, bad)
     torch.cuda.synchronize()
     assert int(bad) == 0 and s.sk.status() == 0
     s.sk.close()
 
 
-def test_another_context_on_the_same_stream(B):
-    s, bad = Selection(B, 2), torch.zeros((), dtype=torch.int64, device="cuda")
+@ROWS
+def test_another_context_on_the_same_stream(B, E, kernel):
+    s, bad = Selection(B, 2, E, kernel), torch.zeros((), dtype=torch.int64, device="cuda")
     n2, k2 = 16500, 40                                           # short selections from candidate lists, which release early
     sk = B.SageKV(8, 2, 128, 1, max_ctx=n2, max_len=4 + 4 * k2 + 8)
     sk.set_select_hint(2, 4 * k2)
