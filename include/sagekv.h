@@ -307,7 +307,9 @@ int sagekv_select_topk(sagekv_ctx *ctx, const float *scores, int64_t scores_row_
  *           histogram of the maxima of 4096 groups of that row's scores and four
  *           tag words (516 32-bit words), and sagekv_select_compact takes its
  *           first threshold bound from that histogram instead of a pass over
- *           the scores.  It verifies the outcome, so scores changed in between,
+ *           the scores (rows of up to 16384 scores it may read whole instead,
+ *           where that is the faster way: few rows, or few kept scores of each).
+ *           It verifies the outcome, so scores changed in between,
  *           or any other content of those words, still select correctly, only
  *           slower.  The caller must give both calls a row stride of at least
  *           sagekv_scores_row_stride() and a buffer that spans

@@ -22,10 +22,9 @@
 //      tie-break (lowest positions win).
 //   4. a kept candidate's output slot is the number of kept candidates before it in the list (one prefix sum):
 //      ascending positions.  Each CTA writes and gathers an even share of the slots.
-// General path (k_q large, tiny rows, or more candidates than the buffers hold, e.g. a row of equal
-// scores): three-digit radix select (11 + 11 + 10 bits) with histograms merged in CTA 0's shared memory by
-// distributed-shared-memory atomics, then a ballot/popcount ranking in row order; launches known to need it from the start have
-// a kernel of their own (select_general_kernel).
+// General path (more candidates than the buffers hold, e.g. a row of equal scores): three-digit radix select (11 + 11 + 10 bits)
+// with histograms merged in CTA 0's shared memory by distributed-shared-memory atomics, then a ballot/popcount ranking in row
+// order; launches known not to take the fast one (k_q large) have a kernel of their own (select_general_kernel).
 // The rows on a CTA's list are then copied into the head's segment of the reduced cache (general path: the
 // CTA that owns a kept element copies it), together with a share of the KV head's sink, recent and last rows.
 #include <cooperative_groups.h>
@@ -1415,13 +1414,18 @@ cudaError_t launch_score_finalize_candidates(const ScoreParams &sp, cudaStream_t
 
 cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t stream) {
   const bool select = p.k_q > 0 && p.E > 0;
-  const int n_rows = select ? p.B * p.H_q : 0;
+  if (!select) {                                         // (the sink, recent and last rows are all there is to copy)
+    SelectParams pl = p;
+    pl.pdl = 0;
+    return launch_copy_static(pl, n_sm, stream, true);
+  }
+  const int n_rows = p.B * p.H_q;
   // The rows may carry the group maxima of the score step (see common.cuh): then the threshold bound costs no
   // pass over the data, the slice is read straight from global memory (no staging: it is needed once), and with
   // many rows smaller clusters pay, because two CTAs per SM times the SM count is all that runs at once.
-  const bool list = select && p.list && list_applies(p.E, p.k_q, p.row_stride);
-  const bool sketch = list || (select && p.sketch && sketch_fits(p.E, p.row_stride));   // both read the row unstaged, if at all
-  if (select && !list && short_rows_apply(p, n_sm, sketch)) return launch_select_short(p, n_sm, stream);
+  const bool list = p.list && list_applies(p.E, p.k_q, p.row_stride);
+  const bool sketch = list || (p.sketch && sketch_fits(p.E, p.row_stride));   // both read the row unstaged, if at all
+  if (!list && short_rows_apply(p, n_sm, sketch)) return launch_select_short(p, n_sm, stream);
   // Cluster size, at most 8 CTAs (the portable limit).
   int cs = 1;
   const int n_static = p.Kc != nullptr ? p.S + p.R + 1 : 0;   // sink, recent and last rows per KV head
@@ -1429,36 +1433,34 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   if (ahead) {
     // From a candidate list nothing but the gather scales with the cluster: a CTA takes up to 128 rows (one round of
     // its 16 warps), and small launches leave room for the next launch's CTAs to run ahead (sagekv_set_select_overlap).
-    while (cs < kMaxCluster && (int64_t)cs * 2048 < p.E && (p.k_q + cs - 1) / cs > 128) cs <<= 1;
+    while (cs < kMaxCluster && (p.k_q + cs - 1) / cs > 128) cs <<= 1;
     ahead = n_static <= kStaticPerWarp * p.G * cs * kSelWarps;            // (more static rows are copied beside: see below)
     if (!ahead) cs = 1;
   }
   if (!ahead && sketch) {
-    while (cs < kMaxCluster && (int64_t)cs * 2048 < p.E && (int64_t)n_rows * cs * 2 <= 2 * (int64_t)n_sm) cs <<= 1;
+    while (cs < kMaxCluster && (int64_t)n_rows * cs * 2 <= 2 * (int64_t)n_sm) cs <<= 1;
   } else if (!ahead) {
     // Slices of at most 16384 scores (one iteration of the passes, and two staged slices fit on an SM), as many CTAs as
     // the prefilter wants thread maxima for k_q, and beyond that only what brings one CTA to every SM: more would not shorten
-    // the chain of block-wide steps that bounds short rows (us per launch with clusters of 8 / 4 / 2: 32 rows x
-    // 16251 14.9 / 11.8 / 12.6, 64 x 25236 with k_q = 1024 52.4 / 40.9 / 62.0, 128 x 6143 with k_q = 512 72.4 / 49.2 / 39.0,
+    // the chain of block-wide steps (us per launch with clusters of 8 / 4 / 2: 64 rows x 25236 with k_q = 1024 52.4 / 40.9 / 62.0,
     // 128 x 59867 60.7 / 39.6 / 41.6, 32 x 130939 18.6 / 18.6 / 26.0).
-    while (cs < kMaxCluster && (int64_t)cs * 512 < p.E &&
+    while (cs < kMaxCluster &&
            ((int64_t)cs * 4 * 8 * kSelThreads < p.E || 2 * (int64_t)p.k_q > (int64_t)cs * kSelThreads || (int64_t)n_rows * cs * 2 <= n_sm))
       cs <<= 1;
   }
   int chunk = (p.E + cs - 1) / cs;
   chunk = (chunk + 3) & ~3;
-  if (chunk < 4) chunk = 4;
-  const int list_cap = chunk < p.k_q ? chunk : (p.k_q > 0 ? p.k_q : 1);
+  const int list_cap = chunk < p.k_q ? chunk : p.k_q;
   // the prefilter needs at least 2*k_q thread maxima; its buffers hold 1.5*k_q + 256 candidates
   // (and its per-row hit table, kept where the candidate copies go later, holds 16 iterations of 4096 vectors)
-  const int try_fast = select && chunk <= 16 * 8 * kSelThreads * 4 &&
+  const int try_fast = chunk <= 16 * 8 * kSelThreads * 4 &&
                        (2 * (int64_t)p.k_q <= (int64_t)cs * kSelThreads || (sketch && 2 * p.k_q <= kSketchFloats));
   const int cand_cap = try_fast ? (p.k_q + p.k_q / 2 + 256) & ~1 : 0;
   const int share = (p.k_q + cs - 1) / cs;              // slots a CTA writes and gathers on the fast path
   const bool resident = !sketch && select_smem_bytes(chunk, list_cap, cand_cap, share, try_fast != 0, true) <= (size_t)kSelSmemLimit;
   const size_t smem = select_smem_bytes(chunk, list_cap, cand_cap, share, try_fast != 0, resident);
   // the gather list of a large k_q on long slices may not fit: refused here, before the static rows' kernel has written any
-  if (select && smem > (size_t)kSelSmemLimit) return cudaErrorInvalidValue;
+  if (smem > (size_t)kSelSmemLimit) return cudaErrorInvalidValue;
 
   // The sink, recent and last rows: the row clusters copy them along with the kept rows as long as that is at most
   // kStaticPerWarp rows per warp.  More of them (the window is then a large share of the budget) would queue up behind the
@@ -1466,14 +1468,14 @@ cudaError_t launch_select_compact(const SelectParams &p, int n_sm, cudaStream_t 
   // launch along / beside: 64 score rows of 25236, 4097 rows per head, 40.6 / 32.2, 32 of them 30.5 / 23.7; 16 pooled rows of
   // 59862, 138 rows, 23.3 / 25.2; from candidate lists of 131072 tokens, 133 rows 4.5 / 6.6, 505 rows 5.8 / 7.4, 1005 rows,
   // four per warp, 7.4 / 7.8, but 69.2 / 67.6 with the score launch in front.)
-  const bool beside = n_static > 0 && (!select || n_static > kStaticPerWarp * p.G * cs * kSelWarps);
+  const bool beside = n_static > kStaticPerWarp * p.G * cs * kSelWarps;
   // Only launches that start from a candidate list, and copy all rows themselves, are short enough to gain from releasing
   // their successor early: successors scheduled early take bandwidth and SM room from the others.
   SelectParams pl = p;
   if (!list || beside) pl.pdl = 0;
   if (beside) {
-    const cudaError_t e = launch_copy_static(pl, n_sm, stream, !select);
-    if (e != cudaSuccess || !select) return e;
+    const cudaError_t e = launch_copy_static(pl, n_sm, stream, false);
+    if (e != cudaSuccess) return e;
   }
   const int64_t sketch_off = try_fast && sketch && !list ? sketch_offset(p.E) : (int64_t)-1;
   const int64_t list_off = try_fast && list ? sketch_offset(p.E) : (int64_t)-1;
