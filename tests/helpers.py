@@ -1,6 +1,8 @@
 """Helpers shared by the GPU tests: bit views, the kernels' comparison key, and the layout of the hint that
 sagekv_score can leave behind the score rows (one copy, so that the tests cannot drift apart)."""
 
+import re
+
 import numpy as np
 import torch
 
@@ -49,12 +51,29 @@ def hint_of(rows, E):
 
 
 def kernels_of(f):
-    """Names of the kernels that f() launches, in order, demangled, without return type, namespace and parameters."""
-    from torch.profiler import ProfilerActivity, profile
+    """Names of the library's kernels that f() launches, sorted, with their template arguments: f() is run once, then captured into a
+    graph, which is read and not run."""
+    from cuda.bindings import driver as cu
+
+    def ok(result):
+        assert int(result[0]) == 0, result
+        return result[1]
+
     f()                                                           # (what is loaded on first use)
     torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+    graph, names = torch.cuda.CUDAGraph(keep_graph=True), []
+    with torch.cuda.graph(graph):
         f()
-        torch.cuda.synchronize()
-    names = [(e.time_range.start, e.name) for e in prof.events() if e.device_type == torch.autograd.DeviceType.CUDA]
-    return [n.split("sagekv::")[1].split("(")[0] for _, n in sorted(names) if "sagekv::" in n]
+    handle = cu.CUgraph(graph.raw_cuda_graph())
+    n = int(cu.cuGraphGetNodes(handle)[2])
+    for node in ok(cu.cuGraphGetNodes(handle, n))[:n]:
+        if ok(cu.cuGraphNodeGetType(node)) != cu.CUgraphNodeType.CU_GRAPH_NODE_TYPE_KERNEL:
+            continue
+        p = ok(cu.cuGraphKernelNodeGetParams(node))
+        mangled = ok(cu.cuFuncGetName(p.func) if int(p.func) else cu.cuKernelGetName(p.kern)).decode()
+        m = re.match(r"_ZN6sagekv(\d+)", mangled)
+        if m:
+            name, rest = mangled[m.end():m.end() + int(m[1])], mangled[m.end() + int(m[1]):]
+            args = re.findall(r"L([bi])(\d+)E", rest.split("EE")[0] + "E") if rest.startswith("I") else []
+            names.append(name + ("<%s>" % ", ".join({"b0": "false", "b1": "true"}.get(t + v, v) for t, v in args) if args else ""))
+    return sorted(names)
