@@ -163,7 +163,7 @@ struct DeviceInfo {
 cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStream_t stream);
 cudaError_t decode_setup(DeviceInfo *dev);   // one-time, with the device current
 // returns the estimated us of a launch, 0 if there is none; mode: the launch overlap mode
-float decode_geometry(int L, int heads, const DeviceInfo *dev, int mode, int *n_clusters, int *cluster_size,
+float decode_geometry(int L, int heads, int G, const DeviceInfo *dev, int mode, int *n_clusters, int *cluster_size,
                       int *resident_tiles, int *smem_bytes);
 
 // ---- status word -------------------------------------------------------------

@@ -740,9 +740,11 @@ cudaError_t decode_setup(DeviceInfo *dev) {
   return cudaFuncSetAttribute(decode_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)decode_tc_smem_bytes(kTcMaxTiles));
 }
 
-// In modes 0 and 1 launches of this many KV heads keep the older, coarser costs of both kernels: with the newer ones 24 x 2561 rows went from
-// 8.5 (whole) to 9.1 us (streamed) and 32 x 1537 from 7.3 to 7.9.
-constexpr int kDecodeManyHeads = 20;
+// In modes 0 and 1 launches of this many KV heads keep the older, coarser costs of both kernels: two launches' clusters of six, the
+// size that suits most of them, no longer fit on the device together, which the newer ones do not follow (us per launch with the older /
+// newer: 17 x 2557 rows, G = 8, 7.0 / 8.1; 19 x 2557 7.1 / 8.6; 19 x 1021 4.9 / 5.6; 24 x 2561 8.5 / 9.1; but 18 x 4097 11.2 / 10.0; of 2892 launches of
+// 1 to 64 heads timed both ways 55 took over 4 % longer with the newer ones from 20 heads on, 11 from 17 on.)
+constexpr int kDecodeManyHeads = 17;
 
 // Whether all nine warps of a CTA ask for its copies, or the ninth alone.  Sharing takes the copies' issue time off the launch, which
 // counts where they are asked for behind the dependency wait, or late because the predecessor's clusters are in the way (us per launch
@@ -763,7 +765,7 @@ static bool decode_shares_issue(int mode, int ctas, int per_cta, int units, int 
 // computes), which only works if the clusters of two launches fit on the device together, so the cluster sizes
 // are compared by a cost fitted to measurements (below).
 // (15 clusters of 8 whole-SM CTAs fit at once, 22 of 6, 26 of 5, 33 of 4.)
-float decode_geometry(int L, int heads, const DeviceInfo *dev, int mode, int *n_clusters, int *cs, int *per_cta_tiles,
+float decode_geometry(int L, int heads, int G, const DeviceInfo *dev, int mode, int *n_clusters, int *cs, int *per_cta_tiles,
                       int *smem_bytes) {
   const int n_tiles = (L + 15) / 16;
   int c = 1;
@@ -784,10 +786,13 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, int mode, int *n_
         const int cap = resident_capacity(dev->device, cand, per);
         if (cap <= 0) continue;
         // Fitted to every cluster size (4 to 8) at 1 to 48 heads x 129 .. 4097 rows in all overlap modes, G = 4 (us per launch): a time
-        // per tile of a CTA, 0.3 - 0.5 and a time per V tile that waits for a K slot where some do, more where the clusters of
-        // two launches do not fit on the device together, up to as much again as they overfill it; and beside that what moving
-        // the rows takes.  3.4 for the merge through scratch (L = 8193, 1 and 8 heads).  (What these rules choose is on average
-        // 0.2 % slower than the best cluster size or streamed launch of each case in mode 2, 0.9 % in mode 0, 1.3 % in mode 1.)
+        // per tile of a CTA, 0.3 - 0.5 and a time per V tile that waits for a K slot where some do (one warp asking for the copies: less by
+        // 0.7, timed at 12 to 16 heads x 2561 .. 5121 rows), more where the clusters of two launches do not fit on the device together, up
+        // to as much again as they overfill it; beside that what moving the rows takes; and for the merge through scratch a time per query
+        // head, whose results it moves (1 to 24 heads x 5697 .. 12289 rows, G = 1, 4, 8: a fixed 3.4 took one head x 12285 rows, G = 8, to 11.1
+        // in place of 9.2, and kept 2 x 8193, G = 1, from 6.2, at 7.0).  (Over 1716 launches in modes 0 and 1, G = 1 to 8, what these rules and
+        // those for the streamed launches choose is on average 1.1 % slower than the best that could be forced; over 1176 at lengths
+        // and numbers of heads between the fitted ones 1.5 %.)
         const int late = 2 * per > kDecodeSlots ? 2 * per - kDecodeSlots : 0, units = heads * n_try;
         const int waves = (units + cap - 1) / cap;                              // of one launch
         const bool is_long = per > kQkGroup * kDecodeWarps;
@@ -800,10 +805,10 @@ float decode_geometry(int L, int heads, const DeviceInfo *dev, int mode, int *n_
           one = 2.89f + 0.035f * (float)per + (is_long ? 0.26f + 0.056f * (float)late : 0.f) + (over >= 0.f ? 0.31f + 0.59f * over : 0.f);
         } else {
           one = decode_shares_issue(mode, units * cand, per, units, n_try) ? 3.11f + 0.073f * share + (is_long ? 0.49f + 0.04f * (float)late : 0.f)
-                                                                           : 3.f + 0.057f * share + 0.072f * (share > 6.f ? share - 6.f : 0.f);
+                                                                           : 3.f + 0.057f * share + 0.072f * (share > 6.f ? share - 6.f : 0.f) - (is_long ? 0.7f - 0.03f * (float)late : 0.f);
           one += over >= 0.f ? 0.21f + 0.28f * over : 0.f;
         }
-        if (n_try > 1) one += 3.4f;
+        if (n_try > 1) one += many ? 3.4f : (mode == 2 ? 2.2f + 0.35f * (float)G : 2.4f + 0.4f * (float)G);
         one = (float)waves * one + (many ? 0.f : 0.5f * (float)(waves - 1));
         if (many) {
           cost = one;
@@ -899,7 +904,7 @@ static bool make_cache_map(CUtensorMap *map, const uint16_t *base, const DecodeP
 cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStream_t stream) {
   int n_clusters, cs, per_cta, smem, split = 1, heads_per_cta = 1;
   const int mode = p.overlapping ? 2 : p.pdl_mode;
-  const float cost = decode_geometry(p.L, p.B * p.H_kv, &dev, mode, &n_clusters, &cs, &per_cta, &smem);
+  const float cost = decode_geometry(p.L, p.B * p.H_kv, p.G, &dev, mode, &n_clusters, &cs, &per_cta, &smem);
   const bool tc = p.variant == 2 && n_clusters == 1 && per_cta <= kTcMaxTiles;
   // Caches that fill the SMs more than once, and long ones, are streamed; short ones are brought in whole.  (us per
   // launch whole / streamed, overlapping: 8 heads x 2049 rows 4.1 / 4.7, 8 x 8193 11.0 / 9.4, 64 x 2049 17.4 / 13.4,
