@@ -4,17 +4,18 @@
 // Flash-decoding on thread-block clusters.  The L rows of one KV head are cut into 16-row tiles that are
 // dealt evenly, as contiguous ranges, to the CTAs of one cluster.  A CTA brings its K and V tiles into shared
 // memory with tensor copies (one 16-row x 64-column box per request, 128-byte swizzle, completion counted on
-// an mbarrier), issued by a ninth warp that does nothing else, or by all nine (decode_shares_issue).  The staging area has 50 slots of one tile
-// (K or V) each.  All K tiles of the range are resident from the start; so are the V tiles while slots last,
+// an mbarrier), issued by a ninth warp that does nothing else, or by all nine (decode_shares_issue).  The staging area has 50
+// slots of one tile (K or V) each.  All K tiles of the range are resident from the start; so are the V tiles while slots last,
 // and the remaining V tiles take over the K slots as soon as the first product is done.  There is one pass:
 //   S = K Q^T     16 rows x 8 heads per mma, a tile per warp in turn (the scores of all its tiles stay in
 //                 registers).  A fragments come from the swizzled tile with ldmatrix, the query (B fragments)
 //                 sits in registers.
-//   softmax       ONE maximum per head over the whole CTA (two block barriers in all), so nothing is ever
+//   softmax       one maximum per head and warp, over all its tiles (two block barriers in all), so nothing is ever
 //                 rescaled; the weights, rounded to bf16, go to shared memory for all tiles.
 //   O^T = V^T P   split by COLUMNS: warp w accumulates columns 16w..16w+15 of all heads over all rows
-//                 (transposing ldmatrix for V, the weights as B fragments).  The warps' results are
-//                 disjoint, so nothing is exchanged or summed inside the CTA.
+//                 (transposing ldmatrix for V, the weights as B fragments), the rows of each warp's weights by themselves,
+//                 and brings the eight sums to the CTA's maximum.  The warps' results are disjoint, so nothing is
+//                 exchanged inside the CTA.
 // Every head masks the rows of the other heads' segments.  The CTAs of a cluster are merged through
 // distributed shared memory: each warp sends its 16 columns straight from registers into the inbox of the
 // CTA that finishes those columns with asynchronous stores counted on that CTA's barrier (one way, no
@@ -63,7 +64,8 @@ struct DecShared {
   uint32_t tmem_base;                                          // tensor-memory variant: first column of the CTA's allocation
   int pad_[2];
   float warp_m[kDecodeWarps][kMaxGroup];                       // maxima of the warps' rows
-  float warp_l[kDecodeWarps][kMaxGroup];                       // sums of the warps' (rounded) weights
+  float warp_l[kDecodeWarps][kMaxGroup];                       // sums of the warps' (rounded) weights, in units of the CTA's maxima
+  float warp_f[kDecodeWarps][kMaxGroup];                       // what brings a warp's weights to these units
   float2 inbox_ml[kDecodeMaxCluster][kMaxGroup];               // [source CTA][head] (max, sum)
   float inbox_o[(kHeadDim + 4 * kDecodeMaxCluster) * kMaxGroup];   // [source CTA][my column][head]; cluster size x columns <= 160
 };
@@ -136,7 +138,8 @@ __device__ __forceinline__ void bar_sync(int id, int n_threads) {
 
 // n_slots: slots of this launch's staging area (min(2 * most tiles of a CTA, kDecodeSlots)).
 // kLong: a CTA may have more tiles than half the slots (part of V arrives late, a warp may have up to six tiles in
-// the first product); false keeps the common case free of that.
+// the first product); false keeps the common case free of that.  kShared: all nine warps ask for the copies at the start, each for
+// a ninth of the boxes (the bytes to expect are set before they do); late V tiles are the ninth warp's in any case.
 template <bool kLong, bool kShared>
 __global__ void __launch_bounds__(kDecodeThreads, 1)
 decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -447,21 +450,10 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
     wm1 = fmaxf(wm1, __shfl_xor_sync(0xffffffffu, wm1, o));
   }
   if (g == 0) { sh.warp_m[warp][h0] = wm0; sh.warp_m[warp][h1] = wm1; }
-  bar_sync(1, kDecodeThreads);   // A: the maxima are complete, and nobody reads a K slot any more (the copy warp refills them)
-
-  float M0, M1;                  // maxima of heads 2c, 2c+1 over the CTA's rows (log2 units)
-  {
-    float a0[kDecodeWarps], a1[kDecodeWarps];
-#pragma unroll
-    for (int w = 0; w < kDecodeWarps; ++w) { a0[w] = sh.warp_m[w][h0]; a1[w] = sh.warp_m[w][h1]; }
-#pragma unroll
-    for (int s2 = kDecodeWarps / 2; s2 > 0; s2 >>= 1)   // a tree, not a chain
-#pragma unroll
-      for (int w = 0; w < s2; ++w) { a0[w] = fmaxf(a0[w], a0[w + s2]); a1[w] = fmaxf(a1[w], a1[w + s2]); }
-    M0 = a0[0]; M1 = a1[0];
-  }
-  SAGEKV_STAMP_AFTER(4, M0 + M1);
-  const float s0 = M0 == -INFINITY ? 0.f : M0, s1 = M1 == -INFINITY ? 0.f : M1;
+  // Each warp's weights are taken relative to its own maximum, which so gets a weight of exactly 1: with one maximum for all rows of the
+  // CTA the largest weights of seven warps were rounded too, and the outputs further from 64-bit ones (relative 2.18e-3, now and in
+  // the streamed kernel 2.0e-3, at 16 heads x 2049 rows, G = 7; the bf16 output alone is 1.7e-3).
+  const float s0 = wm0 == -INFINITY ? 0.f : wm0, s1 = wm1 == -INFINITY ? 0.f : wm1;
   // the weights enter the second product as bf16: one word per (tile, head, row pair g: rows 2g and 2g + 1);
   // their sums per head are taken from the rounded values, so that numerator and denominator agree
   float ls0 = 0.f, ls1 = 0.f;
@@ -485,7 +477,25 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
     ls0 += __shfl_xor_sync(0xffffffffu, ls0, o);
     ls1 += __shfl_xor_sync(0xffffffffu, ls1, o);
   }
-  if (g == 0) { sh.warp_l[warp][h0] = ls0; sh.warp_l[warp][h1] = ls1; }
+  bar_sync(1, kDecodeThreads);   // A: the maxima are complete, and nobody reads a K slot any more (the copy warp refills them)
+
+  float M0, M1;                  // maxima of heads 2c, 2c+1 over the CTA's rows (log2 units)
+  {
+    float a0[kDecodeWarps], a1[kDecodeWarps];
+#pragma unroll
+    for (int w = 0; w < kDecodeWarps; ++w) { a0[w] = sh.warp_m[w][h0]; a1[w] = sh.warp_m[w][h1]; }
+#pragma unroll
+    for (int s2 = kDecodeWarps / 2; s2 > 0; s2 >>= 1)   // a tree, not a chain
+#pragma unroll
+      for (int w = 0; w < s2; ++w) { a0[w] = fmaxf(a0[w], a0[w + s2]); a1[w] = fmaxf(a1[w], a1[w + s2]); }
+    M0 = a0[0]; M1 = a1[0];
+  }
+  SAGEKV_STAMP_AFTER(4, M0 + M1);
+  if (g == 0) {
+    const float f0 = M0 == -INFINITY ? 0.f : fast_exp2(wm0 - M0), f1 = M1 == -INFINITY ? 0.f : fast_exp2(wm1 - M1);
+    sh.warp_f[warp][h0] = f0; sh.warp_f[warp][h1] = f1;
+    sh.warp_l[warp][h0] = ls0 * f0; sh.warp_l[warp][h1] = ls1 * f1;
+  }
   bar_sync(2, kConsumerThreads);   // B: the weights are in shared memory (and a patched early V row is visible)
   SAGEKV_STAMP(5);
   // The (max, sum) pairs of the CTA go to every CTA of the cluster now, ahead of the second product, with
@@ -505,45 +515,49 @@ decode_attn_kernel(const DecodeParams p, const __grid_constant__ CUtensorMap map
   }
 
   // ---- O^T = V^T P: columns 16*warp .. +15 over all rows, the early V tiles first ----
-  // A B fragment is two of the weight words (rows 2c, 2c+1 and 2c+8, 2c+9 of head g).  Six tiles per step, each on an
-  // accumulator chain of its own, all fragments requested before the mmas.  (An mma's result takes about 130
-  // cycles: the sums of the weights used to come from a second mma per tile against a fragment of ones, on two
-  // chains eleven links long, and those chains alone took 0.75 us; they are summed in registers now.)
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};    // O^T: (col_a, h0) (col_a, h1) (col_b, h0) (col_b, h1)
-  float xc[5][4];
+  // A B fragment is two of the weight words (rows 2c, 2c+1 and 2c+8, 2c+9 of head g).  Eight tiles per step, one of each warp's in
+  // the first product on an accumulator chain of its own, which is brought to the CTA's maxima at the end; all fragments
+  // requested before the mmas.  (An mma's result takes about 130 cycles: the sums of the weights used to come from a second
+  // mma per tile against a fragment of ones, on two chains eleven links long, and those chains alone took 0.75 us; they are
+  // summed in registers now.)
+  float xc[kDecodeWarps][4];              // O^T of warp u's rows: (col_a, h0) (col_a, h1) (col_b, h0) (col_b, h1)
 #pragma unroll
-  for (int u = 0; u < 5; ++u) xc[u][0] = xc[u][1] = xc[u][2] = xc[u][3] = 0.f;
-  auto second_product = [&](int t_lo, int t_hi) {
-    for (int t6 = t_lo; t6 < t_hi; t6 += 6) {
-      uint32_t va[6][4], pb[6][2];
+  for (int u = 0; u < kDecodeWarps; ++u) xc[u][0] = xc[u][1] = xc[u][2] = xc[u][3] = 0.f;
+  auto eight_tiles = [&](int t8, int t_hi, bool late) {  // of tiles [t8, t8 + 8) those below t_hi, and with `late` those that came late
+    uint32_t va[kDecodeWarps][4], pb[kDecodeWarps][2];
 #pragma unroll
-      for (int u = 0; u < 6; ++u) {
-        if (t6 + u < t_hi) {
-          ldmatrix_x4_trans(stage + (uint32_t)(v_slot(t6 + u) * kSlotBytes) + v_off, va[u][0], va[u][1], va[u][2], va[u][3]);
-          const uint32_t ra = pr_addr + (uint32_t)((t6 + u) * kPTileWords * 4);
-          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(pb[u][0]) : "r"(ra));
-          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(pb[u][1]) : "r"(ra + 16));
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 6; ++u) {
-        if (t6 + u < t_hi) {
-          if (u == 0) mma_bf16_16816(acc[0], acc[1], acc[2], acc[3], va[u][0], va[u][1], va[u][2], va[u][3], pb[u][0], pb[u][1]);
-          else mma_bf16_16816(xc[u - 1][0], xc[u - 1][1], xc[u - 1][2], xc[u - 1][3], va[u][0], va[u][1], va[u][2], va[u][3], pb[u][0], pb[u][1]);
-        }
+    for (int u = 0; u < kDecodeWarps; ++u) {
+      if (t8 + u < t_hi && (!late || t8 + u >= n_early)) {
+        ldmatrix_x4_trans(stage + (uint32_t)(v_slot(t8 + u) * kSlotBytes) + v_off, va[u][0], va[u][1], va[u][2], va[u][3]);
+        const uint32_t ra = pr_addr + (uint32_t)((t8 + u) * kPTileWords * 4);
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(pb[u][0]) : "r"(ra));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(pb[u][1]) : "r"(ra + 16));
       }
     }
+#pragma unroll
+    for (int u = 0; u < kDecodeWarps; ++u)
+      if (t8 + u < t_hi && (!late || t8 + u >= n_early))
+        mma_bf16_16816(xc[u][0], xc[u][1], xc[u][2], xc[u][3], va[u][0], va[u][1], va[u][2], va[u][3], pb[u][0], pb[u][1]);
   };
   if (n_early > 0 && !mbar_wait(vbar_e, 0u)) timed_out = true;
-  second_product(0, n_early);
+  for (int t8 = 0; t8 < n_early; t8 += kDecodeWarps) eight_tiles(t8, n_early, false);
   if (kLong && n_late > 0) {                             // (the same for every thread of the CTA)
     if (!mbar_wait(vbar_l, 0u)) timed_out = true;
     if (patcher && st >= n_early) patch(true);
     bar_sync(2, kConsumerThreads);                       // a patched late V row is visible
-    second_product(n_early, n);
+    for (int t8 = n_early & ~(kDecodeWarps - 1); t8 < n; t8 += kDecodeWarps) eight_tiles(t8, n, true);
   }
+  float2 wf[kDecodeWarps];                // the warps' factors, asked for while the last products are on their way
 #pragma unroll
-  for (int e = 0; e < 4; ++e) acc[e] += ((xc[0][e] + xc[1][e]) + (xc[2][e] + xc[3][e])) + xc[4][e];
+  for (int u = 0; u < kDecodeWarps; ++u) wf[u] = *reinterpret_cast<const float2 *>(&sh.warp_f[u][h0]);
+  float acc[4];                           // (col_a, h0) (col_a, h1) (col_b, h0) (col_b, h1)
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    float a[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u] = xc[u][e] * ((e & 1) ? wf[u].y : wf[u].x) + xc[u + 4][e] * ((e & 1) ? wf[u + 4].y : wf[u + 4].x);
+    acc[e] = (a[0] + a[1]) + (a[2] + a[3]);
+  }
   if (timed_out) atomicOr(p.status, kStatusWaitTimeout);
   SAGEKV_STAMP_AFTER(6, acc[0] + acc[1] + acc[2] + acc[3]);
 
