@@ -921,8 +921,7 @@ cudaError_t launch_decode(const DecodeParams &p, const DeviceInfo &dev, cudaStre
   const float cost = decode_geometry(p.L, p.B * p.H_kv, p.G, &dev, mode, &n_clusters, &cs, &per_cta, &smem);
   const bool tc = p.variant == 2 && n_clusters == 1 && per_cta <= kTcMaxTiles;
   // Caches that fill the SMs more than once, and long ones, are streamed; short ones are brought in whole.  (us per
-  // launch whole / streamed, overlapping: 8 heads x 2049 rows 4.1 / 4.7, 8 x 8193 11.0 / 9.4, 64 x 2049 17.4 / 13.4,
-  // 256 x 2049 84.8 / 42.8)
+  // launch whole / streamed, overlapping: 8 heads x 2049 rows 3.9 / 4.7, 8 x 8193 10.8 / 8.5, 16 x 8193 21.0 / 13.1, 256 x 2049 84.8 / 42.8)
   const float stream_cost = tc ? 0.f : stream_geometry(p.L, p.B * p.H_kv, p.G, dev, mode, &split, &heads_per_cta);
   const bool streamed = stream_cost > 0.f && cost > 0.f && stream_cost < cost;
   CUtensorMap map_k, map_v;
